@@ -5,10 +5,15 @@
 // shuffles.  Every reduction uses a grid size that depends only on the
 // vector length and the device's multiprocessor count and sums in a fixed
 // order, so results are bit-reproducible on a given device.
+#include <cooperative_groups.h>
+
 #include <atomic>
 #include <cmath>
 
+#include "cluster.h"
 #include "kernels.h"
+
+namespace cg = cooperative_groups;
 
 namespace chnss {
 namespace {
@@ -1029,33 +1034,162 @@ __global__ void k_pcg_p(long n, const double *rzn, const double *rzo, const doub
 }
 
 // --------------------------------------------------------------------------
-// coarse grid
+// coarse grid: dense copies, one block per (node) row
 __global__ void k_dense_csr(int nrows, const int *rowptr, const int *col, const double *val, double add_all,
                             double *dense) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= nrows) return;
-  for (int c = 0; c < nrows; ++c) dense[(long)r * nrows + c] = add_all;
-  for (int k = rowptr[r]; k < rowptr[r + 1]; ++k) dense[(long)r * nrows + col[k]] += val[k];
+  const int r = blockIdx.x;
+  double *row = dense + (long)r * nrows;
+  for (int c = threadIdx.x; c < nrows; c += blockDim.x) row[c] = add_all;
+  __syncthreads();
+  for (int k = rowptr[r] + threadIdx.x; k < rowptr[r + 1]; k += blockDim.x) row[col[k]] += val[k];
 }
 __global__ void k_dense_bsr2(int nrows, const int *rowptr, const int *col, const double *val, double *dense) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= nrows) return;
+  const int r = blockIdx.x;
   const int n = 2 * nrows;
-  for (int c = 0; c < n; ++c) {
-    dense[(long)(2 * r) * n + c] = 0.0;
-    dense[(long)(2 * r + 1) * n + c] = 0.0;
-  }
-  for (int k = rowptr[r]; k < rowptr[r + 1]; ++k) {
+  double *row = dense + (long)(2 * r) * n;
+  for (int c = threadIdx.x; c < 2 * n; c += blockDim.x) row[c] = 0.0;
+  __syncthreads();
+  for (int k = rowptr[r] + threadIdx.x; k < rowptr[r + 1]; k += blockDim.x) {
     const int c = 2 * col[k];
-    dense[(long)(2 * r) * n + c] = val[4L * k];
-    dense[(long)(2 * r) * n + c + 1] = val[4L * k + 1];
-    dense[(long)(2 * r + 1) * n + c] = val[4L * k + 2];
-    dense[(long)(2 * r + 1) * n + c + 1] = val[4L * k + 3];
+    row[c] = val[4L * k];
+    row[c + 1] = val[4L * k + 1];
+    row[n + c] = val[4L * k + 2];
+    row[n + c + 1] = val[4L * k + 3];
   }
 }
 
+// Gauss-Jordan inverse with partial pivoting of a (row-major) into inv for
+// n <= kCoarseDenseMax, by one cluster of kInvCtas blocks.  It runs in every
+// step's setup, where one block (k_dense_invert below) is bound by its
+// multiprocessor's FP64 pipe (2 n^3 multiply-adds at two a clock): 1.43 ms
+// for 98 rows, 30.1 ms for 242.  Here the columns of [a | inv] are dealt to
+// the blocks in turn and stay in shared memory, column-major, so the pipe of
+// every multiprocessor of the cluster works and only pivot column c + 1 is
+// pushed to the others each step (double buffered, one cluster barrier a
+// step).  Every block finds the pivot from its own copy of the column.
+// Columns that are still (or already) unit vectors are left out: their
+// pivot-row entry is zero.  Entry by entry the operations of k_dense_invert.
+// The cluster barrier and the pivot's division now bound the step.
+constexpr int kInvCtas = 16;
+constexpr int kInvThreads = 512;
+static_assert(2 * kCoarseDenseMax / kInvCtas <= 32, "one warp handles a block's columns");
+struct InvSmem {
+  double col[2][kCoarseDenseMax];                     // pivot column, current and next
+  double prow[2 * kCoarseDenseMax / kInvCtas];        // pivot row of the block's columns
+  int used[kCoarseDenseMax];                          // original rows taken as pivots
+  int orig[kCoarseDenseMax];                          // original row at each position
+  int act[2 * kCoarseDenseMax / kInvCtas];            // the block's columns with work in this step
+  int nact, piv;
+};
+inline size_t inv_smem_bytes(int n) {
+  const int lc = (n + kInvCtas - 1) / kInvCtas;
+  return sizeof(InvSmem) + (size_t)2 * lc * n * sizeof(double);
+}
+__global__ void __launch_bounds__(kInvThreads) k_dense_invert_cluster(int n, const double *__restrict__ a,
+                                                                      double *__restrict__ inv, int *status) {
+  extern __shared__ __align__(16) unsigned char raw[];
+  InvSmem &S = *reinterpret_cast<InvSmem *>(raw);
+  double *W = reinterpret_cast<double *>(raw + sizeof(InvSmem));   // [2 lc][n]: a columns, then inv columns
+  cg::cluster_group cl = cg::this_cluster();
+  const int me = (int)cl.block_rank(), tid = threadIdx.x;
+  const int lc = (n + kInvCtas - 1) / kInvCtas;
+  for (int t = tid; t < lc * n; t += kInvThreads) {
+    const int r = t / lc, j = t % lc, q = j * kInvCtas + me;
+    W[j * n + r] = q < n ? a[(long)r * n + q] : 0.0;
+    W[(lc + j) * n + r] = r == q ? 1.0 : 0.0;
+  }
+  for (int r = tid; r < n; r += kInvThreads) {
+    S.col[0][r] = a[(long)r * n];
+    S.used[r] = 0;
+    S.orig[r] = r;
+  }
+  bool zero = false;
+  cl.sync();
+  for (int c = 0; c < n; ++c) {
+    double *cb = S.col[c & 1];
+    if (tid < 32) {   // pivot: largest magnitude, first row among equals; then this step's columns
+      double best = -1.0;
+      int bi = c;
+      for (int r = c + tid; r < n; r += 32) {
+        const double v = fabs(cb[r]);
+        if (v > best) { best = v; bi = r; }
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        const double v2 = __shfl_xor_sync(0xffffffffu, best, o);
+        const int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (v2 > best || (v2 == best && i2 < bi)) { best = v2; bi = i2; }
+      }
+      if (best == 0.0) zero = true;
+      if (tid == 0) {
+        S.piv = bi;
+        const int t = S.orig[bi];
+        S.orig[bi] = S.orig[c];
+        S.orig[c] = t;
+        S.used[t] = 1;
+      }
+      __syncwarp();
+      int na = 0;   // the next pivot column first, so that it can leave early
+      for (int j0 = 0; j0 < 2 * lc; j0 += 32) {
+        const int j = j0 + tid, q = (j < lc ? j : j - lc) * kInvCtas + me;
+        const bool on = j < 2 * lc && q < n && (j < lc ? q > c : S.used[q] != 0);
+        const unsigned m = __ballot_sync(0xffffffffu, on);
+        if (on) S.act[na + __popc(m & ((1u << tid) - 1u))] = j;
+        na += __popc(m);
+      }
+      if (tid == 0) S.nact = na;
+    }
+    __syncthreads();
+    const int p = S.piv, na = S.nact;
+    const double d = cb[p];
+    double cc = 0.0;
+    if (tid < 32) {   // swap rows c and p (in every column), scale the pivot row
+      if (tid < 2 * lc) {
+        double *w = W + tid * n;
+        const double x = w[p];
+        w[p] = w[c];
+        w[c] = x;
+      }
+      __syncwarp();
+      if (tid < na) {
+        double *w = W + S.act[tid] * n;
+        const double v = w[c] / d;
+        w[c] = v;
+        S.prow[tid] = v;
+      }
+    }
+    if (tid == kInvThreads - 1) cc = cb[c];
+    __syncthreads();
+    if (tid == kInvThreads - 1) cb[p] = cc;
+    __syncthreads();
+    const int rows = (n + 31) / 32 * 32, groups = kInvThreads / rows;
+    const int g = tid / rows, r = tid % rows;
+    const bool mine = c + 1 < n && (c + 1) % kInvCtas == me;   // act[0] is column c + 1 then
+    if (g < groups && r < n && r != c) {
+      const double f = cb[r];
+      for (int k = g; k < na; k += groups) {
+        double *w = W + S.act[k] * n;
+        w[r] -= f * S.prow[k];
+      }
+    }
+    if (mine) {
+      __syncthreads();
+      const double *w = W + ((c + 1) / kInvCtas) * n;
+      for (int t = tid; t < n * kInvCtas; t += kInvThreads)
+        cl.map_shared_rank(&S.col[(c + 1) & 1][0], t / n)[t % n] = w[t % n];
+    }
+    cl.sync();
+  }
+  for (int t = tid; t < lc * n; t += kInvThreads) {
+    const int r = t / lc, j = t % lc, q = j * kInvCtas + me;
+    if (q < n) inv[(long)r * n + q] = W[(lc + j) * n + r];
+  }
+  if (me == 0 && tid == 0) *status = zero ? 1 : 0;
+}
+
 // Gauss-Jordan inverse with partial pivoting of a (n x n, row-major,
-// destroyed) into inv; one CTA.  status = 1 on an exactly zero pivot.
+// destroyed) into inv; one CTA.  status = 1 on an exactly zero pivot.  For
+// the sizes above kCoarseDenseMax (the pressure Laplacian's coarsest level,
+// inverted once per context).
 __global__ void k_dense_invert(int n, double *a, double *inv, int *status) {
   __shared__ int piv;
   __shared__ double sv[TPB];
@@ -2339,14 +2473,22 @@ void pcg_update_p(long n, const double *rzn, const double *rzo, const double *z,
 }
 
 void coarse_dense_csr(const Pattern &P, const double *val, double add_all, double *dense, cudaStream_t s) {
-  k_dense_csr<<<nblocks(P.nrows, 128), 128, 0, s>>>(P.nrows, P.rowptr, P.col, val, add_all, dense);
+  k_dense_csr<<<P.nrows, 128, 0, s>>>(P.nrows, P.rowptr, P.col, val, add_all, dense);
   CHNSS_LAUNCH_CK();
 }
 void coarse_dense_bsr2(const Pattern &P, const double *val, double *dense, cudaStream_t s) {
-  k_dense_bsr2<<<nblocks(P.nrows, 128), 128, 0, s>>>(P.nrows, P.rowptr, P.col, val, dense);
+  k_dense_bsr2<<<P.nrows, 128, 0, s>>>(P.nrows, P.rowptr, P.col, val, dense);
   CHNSS_LAUNCH_CK();
 }
 void dense_invert(int n, double *a, double *inv, int *status, cudaStream_t s) {
+  if (n <= kCoarseDenseMax) {
+    constexpr size_t most = sizeof(InvSmem) + 2 * (kCoarseDenseMax / kInvCtas) * kCoarseDenseMax * sizeof(double);
+    allow_cluster<k_dense_invert_cluster>(most);
+    launch_cluster(k_dense_invert_cluster, kInvCtas, 1, kInvThreads, inv_smem_bytes(n), s, n, (const double *)a, inv,
+                   status);
+    CHNSS_LAUNCH_CK();
+    return;
+  }
   k_dense_invert<<<1, TPB, 0, s>>>(n, a, inv, status);
   CHNSS_LAUNCH_CK();
 }
