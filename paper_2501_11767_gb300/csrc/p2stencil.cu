@@ -1,0 +1,437 @@
+// P2 velocity stencil kernels (see p2stencil.h).
+#include "p2stencil.h"
+
+namespace chnss {
+namespace {
+
+constexpr int TPB = 256;
+
+// couplings of the four node types, in CSR (ascending lattice) order
+__host__ __device__ constexpr int slot_base(int ty) { return ty == 0 ? 0 : 10 + 9 * ty; }
+__host__ __device__ constexpr int slot_count(int ty) { return ty == 0 ? 19 : 9; }
+struct SlotTable {
+  signed char di[kP2Slots], dj[kP2Slots];
+};
+__host__ __device__ constexpr SlotTable slot_table() {
+  return {{-2, -1, 0, -2, -1, 0, 1, -2, -1, 0, 1, 2, -1, 0, 1, 2, 0, 1, 2,   // vertex
+           -1, -1, 0, -1, 0, 1, 0, 1, 1,                                     // horizontal edge
+           -2, -1, 0, -1, 0, 1, 0, 1, 2,                                     // vertical edge
+           -1, 0, 1, -1, 0, 1, -1, 0, 1},                                    // diagonal edge
+          {-2, -2, -2, -1, -1, -1, -1, 0, 0, 0, 0, 0, 1, 1, 1, 1, 2, 2, 2,
+           -2, -1, -1, 0, 0, 0, 1, 1, 2,
+           -1, -1, -1, 0, 0, 0, 1, 1, 1,
+           -1, -1, -1, 0, 0, 0, 1, 1, 1}};
+}
+constexpr SlotTable kSlots = slot_table();
+
+// type of the node at lattice parity (pi, pj)
+__host__ __device__ constexpr int type_of(int pi, int pj) { return (pi & 1) + 2 * (pj & 1); }
+// slot of the row of slot k's column that points back (its transposed entry)
+constexpr int back_slot(int ty, int k) {
+  const int di = kSlots.di[slot_base(ty) + k], dj = kSlots.dj[slot_base(ty) + k];
+  const int tc = type_of((ty & 1) + (di & 1), (ty >> 1) + (dj & 1));
+  for (int q = 0; q < slot_count(tc); ++q)
+    if (kSlots.di[slot_base(tc) + q] == -di && kSlots.dj[slot_base(tc) + q] == -dj) return q;
+  return -1;
+}
+struct BackTable {
+  signed char k[kP2Slots];
+};
+constexpr BackTable make_back() {
+  BackTable b{};
+  for (int ty = 0; ty < 4; ++ty)
+    for (int k = 0; k < slot_count(ty); ++k) b.k[slot_base(ty) + k] = (signed char)back_slot(ty, k);
+  return b;
+}
+constexpr BackTable kBack = make_back();
+constexpr bool back_complete() {
+  for (int k = 0; k < kP2Slots; ++k)
+    if (kBack.k[k] < 0) return false;
+  return true;
+}
+static_assert(back_complete(), "the stencil is structurally symmetric");
+
+__constant__ SlotTable c_slots = kSlots;
+__constant__ BackTable c_back = kBack;
+
+__device__ __forceinline__ bool prescribed(int I, int J, int m, int open) {
+  return I <= 0 || J <= 0 || I >= m - 1 || (open ? J >= m : J >= m - 1);
+}
+
+template <typename T> struct V2;
+template <> struct V2<float> { using type = float2; };
+template <> struct V2<double> { using type = double2; };
+template <typename T>
+__device__ __forceinline__ typename V2<T>::type mk(T x, T y) {
+  typename V2<T>::type v;
+  v.x = x;
+  v.y = y;
+  return v;
+}
+__device__ __forceinline__ float2 load_pair(const float *p) { return __ldg(reinterpret_cast<const float2 *>(p)); }
+__device__ __forceinline__ double2 load_pair(const double *p) { return __ldg(reinterpret_cast<const double2 *>(p)); }
+__device__ __forceinline__ float2 load_pair(const __nv_bfloat16 *p) {
+  return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p));
+}
+__device__ __forceinline__ float fma_t(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_t(double a, double b, double c) { return fma(a, b, c); }
+template <typename T> __device__ __forceinline__ T from_double(double x) { return (T)x; }
+template <> __device__ __forceinline__ __nv_bfloat16 from_double<__nv_bfloat16>(double x) { return __double2bfloat16(x); }
+
+template <typename T>
+struct Coef {
+  T c[2 * (kP2Slots + kP2TopSlots)];
+};
+struct Args {
+  const void *b, *w, *dinv;
+  const double *coef, *scale;
+};
+
+// what the sweep's result for one node needs beside its row sums
+template <typename T>
+struct NodeIn {
+  using P = typename V2<T>::type;
+  P b, d, w;
+  T c0 = 0, c1 = 0, c2 = 0;
+  bool has_w = false;
+  __device__ __forceinline__ void load(int mode, int start, long r, T sc, const Args &a, const T *out) {
+    if (mode == SPMV_PLAIN) return;
+    if (mode == SPMV_ADD) {
+      b = reinterpret_cast<const P *>(out)[r];
+      return;
+    }
+    b = static_cast<const P *>(a.b)[r];
+    if (mode == SPMV_RES) return;
+    d = static_cast<const P *>(a.dinv)[r];
+    c0 = (T)a.coef[0];
+    c1 = (T)a.coef[1];
+    c2 = (T)a.coef[2];
+    has_w = start == P2_SECOND || a.w != nullptr;
+    if (start == P2_SECOND) w = mk<T>(sc * d.x * b.x, sc * d.y * b.y);
+    else if (a.w) w = static_cast<const P *>(a.w)[r];
+  }
+  __device__ __forceinline__ P result(int mode, T s0, T s1, P ui) const {
+    if (mode == SPMV_PLAIN) return mk<T>(s0, s1);
+    if (mode == SPMV_RES) return mk<T>(b.x - s0, b.y - s1);
+    if (mode == SPMV_ADD) return mk<T>(b.x + s0, b.y + s1);
+    T v0 = c0 * ui.x + c2 * d.x * (b.x - s0);
+    T v1 = c0 * ui.y + c2 * d.y * (b.y - s1);
+    if (has_w) {
+      v0 += c1 * w.x;
+      v1 += c1 * w.y;
+    }
+    return mk<T>(v0, v1);
+  }
+};
+
+// Fine levels: one cell (its four nodes) a thread.  The 19 neighbours of the
+// vertex are all the cell reads, every value load is one coalesced access of
+// two values, and all loads are independent.
+template <typename T, typename VT, bool OPEN, bool VEC>
+__global__ void __launch_bounds__(kSellMaxBlock, sizeof(T) == 4 ? 2 : 1) k_p2_spmv(int n, long ld, const VT *__restrict__ val,
+                                                           const T *__restrict__ u, T *out, int mode, int start,
+                                                           Args a, const __grid_constant__ Coef<T> cf) {
+  using P = typename V2<T>::type;
+  const int cell = blockIdx.x * blockDim.x + threadIdx.x;
+  const int w1 = n + 1, m = 2 * n + 1;
+  if (cell >= w1 * w1) return;
+  const int j = cell / w1, i = cell - j * w1;
+  P *o2 = reinterpret_cast<P *>(out);
+  const T sc = start != P2_PLAIN ? (T)*a.scale : (T)0;
+  auto iterate = [&](long r) {
+    if (start == P2_FIRST) {
+      const P d = static_cast<const P *>(a.dinv)[r], b = static_cast<const P *>(a.b)[r];
+      return mk<T>(sc * d.x * b.x, sc * d.y * b.y);
+    }
+    if (VEC) return reinterpret_cast<const P *>(u)[r];
+    return mk<T>(u[2 * r], u[2 * r + 1]);
+  };
+  const long r0 = (long)(2 * j) * m + 2 * i;
+  constexpr SlotTable st = slot_table();
+  P x[19];
+#pragma unroll
+  for (int k = 0; k < 19; ++k) {
+    const int I = 2 * i + st.di[k], J = 2 * j + st.dj[k];
+    x[k] = prescribed(I, J, m, OPEN) ? mk<T>(0, 0) : iterate(r0 + st.dj[k] * m + st.di[k]);
+  }
+  auto row = [&](auto tyc) {
+    constexpr int TY = decltype(tyc)::value;
+    constexpr int oi = TY & 1, oj = TY >> 1, base = slot_base(TY), cnt = slot_count(TY);
+    const int I = 2 * i + oi, J = 2 * j + oj;
+    if (I >= m || J >= m) return;
+    const long r = r0 + oj * m + oi;
+    T s0 = 0, s1 = 0;
+    P ui;
+    if (prescribed(I, J, m, OPEN)) {   // identity row
+      ui = iterate(r);
+      s0 = ui.x;
+      s1 = ui.y;
+    } else {
+      const int top = OPEN && TY < 2 && j == n ? kP2Slots : 0;
+#pragma unroll
+      for (int k = 0; k < cnt; ++k) {
+        const int di = oi + st.di[base + k], dj = oj + st.dj[base + k];
+        int xi = 0;
+#pragma unroll
+        for (int q = 0; q < 19; ++q)
+          if (st.di[q] == di && st.dj[q] == dj) xi = q;
+        const P v = load_pair(val + 2 * ((base + k) * ld + cell));
+        const P xk = x[xi];
+        if (di == oi && dj == oj) ui = xk;
+        s0 = fma_t(cf.c[2 * (top + base + k)], xk.y, fma_t((T)v.x, xk.x, s0));
+        s1 = fma_t((T)v.y, xk.y, fma_t(cf.c[2 * (top + base + k) + 1], xk.x, s1));
+      }
+    }
+    NodeIn<T> in;
+    in.load(mode, start, r, sc, a, out);
+    o2[r] = in.result(mode, s0, s1, ui);
+  };
+  row(std::integral_constant<int, 0>());
+  row(std::integral_constant<int, 1>());
+  row(std::integral_constant<int, 2>());
+  row(std::integral_constant<int, 3>());
+}
+
+// Coarse levels (fewer rows than one wave of threads), FP32: 32 cells of one
+// node type (blockIdx.y) a block and KS warps a row, warp q summing entries q,
+// q + KS, ..., the partial sums added in warp order, so that a thread has at
+// most three (KS = 8) dependent blocks.  Latency bound.
+template <typename VT, int KS, bool OPEN>
+__global__ void __launch_bounds__(32 * KS) k_p2_split(int n, long ld, const VT *__restrict__ val,
+                                                      const float *__restrict__ u, float *out, int mode, int start,
+                                                      Args a, const float *__restrict__ tab) {
+  using T = float;
+  using P = float2;
+  __shared__ P part[KS][32];
+  const int lane = threadIdx.x & 31, q = threadIdx.x >> 5, ty = blockIdx.y;
+  const int cell = blockIdx.x * 32 + lane, w1 = n + 1, m = 2 * n + 1;
+  const int j = cell / w1, i = cell - j * w1;
+  const int I = 2 * i + (ty & 1), J = 2 * j + (ty >> 1);
+  const bool live = cell < w1 * w1 && I < m && J < m;
+  const P *u2 = reinterpret_cast<const P *>(u);
+  const T sc = start != P2_PLAIN ? (T)*a.scale : (T)0;
+  auto iterate = [&](long r) {
+    if (start == P2_FIRST) {
+      const P d = static_cast<const P *>(a.dinv)[r], b = static_cast<const P *>(a.b)[r];
+      return mk<T>(sc * d.x * b.x, sc * d.y * b.y);
+    }
+    return u2[r];
+  };
+  const long r = (long)J * m + I;
+  NodeIn<T> in;
+  P ui = mk<T>(0, 0);
+  if (q == 0 && live) {   // the result's operands, requested with the matrix
+    ui = iterate(r);
+    in.load(mode, start, r, sc, a, out);
+  }
+  const bool fixed = live && prescribed(I, J, m, OPEN);
+  T s0 = 0, s1 = 0;
+  if (live && !fixed) {
+    const int base = slot_base(ty), cnt = slot_count(ty), top = OPEN && J == m - 1 ? kP2Slots : 0;
+    constexpr int most = (19 + KS - 1) / KS;
+#pragma unroll
+    for (int t = 0; t < most; ++t) {
+      const int k = base + q + KS * t;
+      if (k < base + cnt) {
+        const int di = c_slots.di[k], dj = c_slots.dj[k];
+        const float2 v = load_pair(val + 2 * (k * ld + cell)), c = load_pair(tab + 2 * (top + k));
+        const float2 x = prescribed(I + di, J + dj, m, OPEN) ? make_float2(0.f, 0.f) : iterate(r + dj * m + di);
+        s0 = fmaf(c.x, x.y, fmaf(v.x, x.x, s0));
+        s1 = fmaf(v.y, x.y, fmaf(c.y, x.x, s1));
+      }
+    }
+  }
+  part[q][lane] = mk<T>(s0, s1);
+  __syncthreads();
+  if (q != 0 || !live) return;
+  if (fixed) {   // identity row
+    s0 = ui.x;
+    s1 = ui.y;
+  } else {
+#pragma unroll
+    for (int p = 1; p < KS; ++p) {
+      s0 += part[p][lane].x;
+      s1 += part[p][lane].y;
+    }
+  }
+  reinterpret_cast<P *>(out)[r] = in.result(mode, s0, s1, ui);
+}
+
+// diagonal values of every block, slot by slot; entry k of a row is its k-th
+// CSR entry (rows with prescribed velocity have none, an open top's rows lack
+// the last ones)
+template <typename VT, bool TRANS>
+__global__ void k_p2_values(int n, int open, long ld, const int *__restrict__ rowptr, const double *__restrict__ A,
+                            VT *__restrict__ out, double *__restrict__ out2) {
+  const int cell = blockIdx.x * TPB + threadIdx.x, k = blockIdx.y;
+  if (cell >= ld) return;
+  const int w1 = n + 1, m = 2 * n + 1, j = cell / w1, i = cell - j * w1;
+  const int ty = k < 19 ? 0 : (k - 10) / 9;
+  const int I = 2 * i + (ty & 1), J = 2 * j + (ty >> 1);
+  const int CI = I + c_slots.di[k], CJ = J + c_slots.dj[k];
+  double2 v = make_double2(0.0, 0.0);
+  if (cell < w1 * w1 && !prescribed(I, J, m, open) && !prescribed(CI, CJ, m, open)) {
+    const int r = TRANS ? CJ * m + CI : J * m + I;
+    const int q = rowptr[r] + (TRANS ? c_back.k[k] : k - slot_base(ty));
+    v = make_double2(A[4L * q], A[4L * q + 3]);
+  }
+  const long e = 2 * (k * ld + cell);
+  out[e] = from_double<VT>(v.x);
+  out[e + 1] = from_double<VT>(v.y);
+  if (out2) *reinterpret_cast<double2 *>(out2 + e) = v;
+}
+
+// the off-diagonal entries of the rows nearest the centre, then a check of
+// every row against them (bad[0] counts the blocks that differ)
+__global__ void k_p2_table(int n, int open, const int *__restrict__ rowptr, const double *__restrict__ A,
+                           double *__restrict__ c) {
+  const int k = threadIdx.x;
+  if (k >= kP2Slots + kP2TopSlots) return;
+  const int m = 2 * n + 1, s = k < kP2Slots ? k : k - kP2Slots;
+  const int ty = s < 19 ? 0 : (s - 10) / 9;
+  c[2 * k] = c[2 * k + 1] = 0.0;
+  const int I = 2 * (n / 2) + (ty & 1), J = k < kP2Slots ? 2 * (n / 2) + (ty >> 1) : 2 * n;
+  if (prescribed(I, J, m, open) || J + c_slots.dj[s] >= m) return;
+  // a coupling to a prescribed node holds zeros: take it from another row of the type
+  int ci = I, cj = J;
+  for (int t = 0; t < n && prescribed(ci + c_slots.di[s], cj + c_slots.dj[s], m, open); ++t) {
+    ci = 2 * t + (ty & 1);
+    for (int v = 0; v < n; ++v) {
+      cj = k < kP2Slots ? 2 * v + (ty >> 1) : 2 * n;
+      if (!prescribed(ci, cj, m, open) && !prescribed(ci + c_slots.di[s], cj + c_slots.dj[s], m, open)) break;
+    }
+  }
+  if (prescribed(ci, cj, m, open) || prescribed(ci + c_slots.di[s], cj + c_slots.dj[s], m, open)) return;
+  const int q = rowptr[cj * m + ci] + s - slot_base(ty);
+  c[2 * k] = A[4L * q + 1];
+  c[2 * k + 1] = A[4L * q + 2];
+}
+__global__ void k_p2_check(int n, int open, const int *__restrict__ rowptr, const int *__restrict__ col,
+                           const double *__restrict__ A, const double *__restrict__ c, int *bad) {
+  const int r = blockIdx.x * TPB + threadIdx.x, m = 2 * n + 1;
+  if (r >= m * m) return;
+  const int I = r % m, J = r / m, ty = type_of(I, J);
+  bool same = true;
+  if (prescribed(I, J, m, open)) {
+    for (int q = rowptr[r]; q < rowptr[r + 1]; ++q) {
+      const double d = col[q] == r ? 1.0 : 0.0;
+      same = same && A[4L * q] == d && A[4L * q + 3] == d && A[4L * q + 1] == 0.0 && A[4L * q + 2] == 0.0;
+    }
+  } else {
+    const int top = J == m - 1 ? kP2Slots : 0;
+    const int len = rowptr[r + 1] - rowptr[r];
+    same = len == (top ? (ty == 0 ? 12 : 6) : slot_count(ty));
+    for (int k = 0; same && k < len; ++k) {
+      const int s = slot_base(ty) + k, q = rowptr[r] + k;
+      const int CI = I + c_slots.di[s], CJ = J + c_slots.dj[s];
+      same = col[q] == CJ * m + CI;
+      const bool off = prescribed(CI, CJ, m, open);
+      same = same && A[4L * q + 1] == (off ? 0.0 : c[2 * (top + s)]) && A[4L * q + 2] == (off ? 0.0 : c[2 * (top + s) + 1]);
+      if (off) same = same && A[4L * q] == 0.0 && A[4L * q + 3] == 0.0;
+    }
+  }
+  if (!same) atomicAdd(bad, 1);
+}
+
+}  // namespace
+
+constexpr int kCount = 2 * (kP2Slots + kP2TopSlots);
+
+bool p2_applies(const Level &L, const P2Table &t, size_t value_size) {
+  return t.ok && (value_size < 8 || sell_warps_bsr2(L.p2.sell) == 1);
+}
+
+P2Table p2_table(Arena &keep, const Level &L, int open_top, const double *A, cudaStream_t s) {
+  P2Table t;
+  Arena ar;
+  double *c = ar.alloc<double>(2 * (kP2Slots + kP2TopSlots));
+  int *bad = ar.alloc<int>(1);
+  CHNSS_CK(cudaMemsetAsync(bad, 0, sizeof(int), s));
+  k_p2_table<<<1, 128, 0, s>>>(L.n, open_top, L.p2.rowptr, A, c);
+  CHNSS_LAUNCH_CK();
+  k_p2_check<<<(L.N2 + TPB - 1) / TPB, TPB, 0, s>>>(L.n, open_top, L.p2.rowptr, L.p2.col, A, c, bad);
+  CHNSS_LAUNCH_CK();
+  int hbad = 0;
+  CHNSS_CK(cudaMemcpyAsync(t.c, c, sizeof(t.c), cudaMemcpyDeviceToHost, s));
+  CHNSS_CK(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
+  CHNSS_CK(cudaStreamSynchronize(s));
+  t.ok = hbad == 0;
+  std::vector<float> f(t.c, t.c + kCount), h(kCount);
+  for (int k = 0; k < kCount; ++k) h[k] = __bfloat162float(__double2bfloat16(t.c[k]));
+  t.d64 = keep.upload(std::vector<double>(t.c, t.c + kCount));
+  t.d32 = keep.upload(f);
+  t.d16 = keep.upload(h);
+  return t;
+}
+
+template <typename VT>
+void p2_values(const Level &L, int open_top, const double *A, bool transposed, VT *out, double *out2, cudaStream_t s) {
+  const long ld = p2_ld(L.n);
+  const dim3 g((unsigned)((ld + TPB - 1) / TPB), kP2Slots);
+  if (transposed) k_p2_values<VT, true><<<g, TPB, 0, s>>>(L.n, open_top, ld, L.p2.rowptr, A, out, out2);
+  else k_p2_values<VT, false><<<g, TPB, 0, s>>>(L.n, open_top, ld, L.p2.rowptr, A, out, out2);
+  CHNSS_LAUNCH_CK();
+}
+template void p2_values<float>(const Level &, int, const double *, bool, float *, double *, cudaStream_t);
+template void p2_values<double>(const Level &, int, const double *, bool, double *, double *, cudaStream_t);
+template void p2_values<__nv_bfloat16>(const Level &, int, const double *, bool, __nv_bfloat16 *, double *, cudaStream_t);
+
+namespace {
+inline bool aligned(const void *p, size_t bytes) { return (reinterpret_cast<uintptr_t>(p) % bytes) == 0; }
+
+template <typename T, typename VT, bool OPEN>
+void launch(const Level &L, int ks, const VT *val, const T *u, T *out, SpmvMode mode, P2Start start, const Args &a,
+            const Coef<T> &cf, const T *tab, cudaStream_t s) {
+  const int cells = (L.n + 1) * (L.n + 1), tpb = L.p2.sell.block, nb = (cells + tpb - 1) / tpb;
+  const long ld = p2_ld(L.n);
+  if (!aligned(u, 2 * sizeof(T))) {   // a caller's solution vector
+    if constexpr (sizeof(T) == 8) {
+      k_p2_spmv<T, VT, OPEN, false><<<nb, tpb, 0, s>>>(L.n, ld, val, u, out, mode, start, a, cf);
+      return;
+    }
+    throw Error{CHNSS_ERR_ARG, "velocity vectors must be aligned to one node"};
+  }
+  if constexpr (sizeof(T) == 4) {
+    const dim3 gs((unsigned)((cells + 31) / 32), 4);
+    switch (ks) {
+      case 2: k_p2_split<VT, 2, OPEN><<<gs, 64, 0, s>>>(L.n, ld, val, u, out, mode, start, a, tab); return;
+      case 4: k_p2_split<VT, 4, OPEN><<<gs, 128, 0, s>>>(L.n, ld, val, u, out, mode, start, a, tab); return;
+      case 8: k_p2_split<VT, 8, OPEN><<<gs, 256, 0, s>>>(L.n, ld, val, u, out, mode, start, a, tab); return;
+    }
+  } else if (ks != 1) {
+    throw Error{CHNSS_ERR_ARG, "FP64 velocity stencil: fine levels only"};
+  }
+  k_p2_spmv<T, VT, OPEN, true><<<nb, tpb, 0, s>>>(L.n, ld, val, u, out, mode, start, a, cf);
+}
+// the table in the precision of the values, on the device and (rounded the
+// same way) as kernel arguments
+const double *device_table(const P2Table &t, const double *) { return t.d64; }
+const float *device_table(const P2Table &t, const float *) { return t.d32; }
+const float *device_table(const P2Table &t, const __nv_bfloat16 *) { return t.d16; }
+double rounded(double x, const double *) { return x; }
+float rounded(double x, const float *) { return (float)x; }
+float rounded(double x, const __nv_bfloat16 *) { return __bfloat162float(__double2bfloat16(x)); }
+}  // namespace
+
+template <typename T, typename VT>
+void p2_spmv(const Level &L, int open_top, const P2Table &tab, const VT *val, const T *u, T *out, SpmvMode mode,
+             const SpmvArgs &a, P2Start start, const double *scale, cudaStream_t s) {
+  for (const void *q : {(const void *)out, a.b, a.w, a.dinv})
+    if (!aligned(q, 2 * sizeof(T))) throw Error{CHNSS_ERR_ARG, "velocity vectors must be aligned to one node"};
+  Coef<T> cf;
+  for (int k = 0; k < kCount; ++k) cf.c[k] = rounded(tab.c[k], val);
+  const T *dt = device_table(tab, val);
+  const Args ka = {a.b, a.w, a.dinv, a.coef, scale};
+  const int ks = sell_warps_bsr2(L.p2.sell);
+  if (open_top) launch<T, VT, true>(L, ks, val, u, out, mode, start, ka, cf, dt, s);
+  else launch<T, VT, false>(L, ks, val, u, out, mode, start, ka, cf, dt, s);
+  CHNSS_LAUNCH_CK();
+}
+template void p2_spmv<float, float>(const Level &, int, const P2Table &, const float *, const float *, float *,
+                                    SpmvMode, const SpmvArgs &, P2Start, const double *, cudaStream_t);
+template void p2_spmv<float, __nv_bfloat16>(const Level &, int, const P2Table &, const __nv_bfloat16 *, const float *,
+                                            float *, SpmvMode, const SpmvArgs &, P2Start, const double *, cudaStream_t);
+template void p2_spmv<double, double>(const Level &, int, const P2Table &, const double *, const double *, double *,
+                                      SpmvMode, const SpmvArgs &, P2Start, const double *, cudaStream_t);
+
+}  // namespace chnss

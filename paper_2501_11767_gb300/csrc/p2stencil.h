@@ -1,0 +1,62 @@
+// The P2 velocity operator of the structured meshes as a stencil over cells.
+//
+// Node types on the once-refined lattice, per cell (i, j), 0 <= i, j <= n:
+// vertices (2i, 2j) with 19 couplings, and the midpoints of horizontal
+// (2i + 1, 2j), vertical (2i, 2j + 1) and diagonal (2i + 1, 2j + 1) edges with
+// 9 each; kDI / kDJ list them in CSR order (46 slots a cell).  Every 2x2 block
+// is s I + eta K_ab: mass and convection act on both components alike, so its
+// off-diagonal entries come from the symmetric gradient alone and are the
+// same for every node of a type (twice over: the open top's nodes see only
+// the elements below them).  A level therefore stores the two diagonal values
+// of each block, at slot * ld + cell, and a table of the off-diagonal ones;
+// columns follow from the cell.  Rows and columns of nodes with prescribed
+// velocity are the identity's and need no values.  A fine sweep moves 92
+// bytes of matrix per node in FP32 where the 2x2-block SELL moves 230.
+#pragma once
+
+#include "kernels.h"
+
+namespace chnss {
+
+constexpr int kP2Slots = 46;
+constexpr int kP2TopSlots = 28;                  // vertex and horizontal slots of the open top's rows
+
+// off-diagonal entries (0,1) and (1,0) by slot; rows on an open top from kP2Slots on
+struct P2Table {
+  double c[2 * (kP2Slots + kP2TopSlots)];
+  // device copies: FP64, rounded to FP32, rounded to BF16 (as FP32)
+  const double *d64 = nullptr;
+  const float *d32 = nullptr, *d16 = nullptr;
+  bool ok = false;                               // every row of the level matches it
+};
+
+inline long p2_ld(int n) { return ((long)(n + 1) * (n + 1) + 31) / 32 * 32; }
+inline long p2_values_count(int n) { return 2 * kP2Slots * p2_ld(n); }   // scalars
+
+// Whether a level with table t takes the stencil for values of value_size
+// bytes: always in FP32 and BF16 (384^2: fine level 31.0 -> 18.0 us a sweep,
+// 192^2 level 12.1 -> 10.9, coarser ones 6.1 -> 4.4-5.1), in FP64 from the
+// size on at which a row is one thread's (n = 241).  Below it an FP64 sweep
+// is bound by its arithmetic and its latencies, and the SELL kernel with
+// several warps a slice is the faster one (128^2: 16.5 against 18.7 us).
+bool p2_applies(const Level &L, const P2Table &t, size_t value_size);
+// Table of the level's constant blocks A (CSR order, 4 values each) and
+// whether all its rows match it (synchronises s); device copies from keep.
+P2Table p2_table(Arena &keep, const Level &L, int open_top, const double *A, cudaStream_t s);
+// Diagonal values of A (or of its transpose) in stencil order; out2 (may be
+// null) receives a second copy in FP64
+template <typename VT>
+void p2_values(const Level &L, int open_top, const double *A, bool transposed, VT *out, double *out2, cudaStream_t s);
+
+// How a Chebyshev sweep (SPMV_CHEB) takes its previous iterates:
+//   P2_PLAIN  u from u, w from args.w (or none)
+//   P2_FIRST  u = *scale dinv b, formed on the fly; no w
+//   P2_SECOND u from u, w = *scale dinv b, formed on the fly
+enum P2Start { P2_PLAIN = 0, P2_FIRST = 1, P2_SECOND = 2 };
+
+// Same row sums, in the same order, as spmv_sell_bsr2 on the level's pattern.
+template <typename T, typename VT>
+void p2_spmv(const Level &L, int open_top, const P2Table &tab, const VT *val, const T *u, T *out, SpmvMode mode,
+             const SpmvArgs &a, P2Start start, const double *scale, cudaStream_t s);
+
+}  // namespace chnss

@@ -149,7 +149,7 @@ void MGHier<T>::init(Arena &ar, int kind_, bool singular_, const std::vector<con
   for (int l = 0; l < nl; ++l) {
     const long nu = (kind == 1 ? 2L : 1L) * pat[l]->nrows;
     n[l] = nu;
-    const long nv = sell_values(l);   // SELL order
+    const long nv = sell_values(l, sizeof(T));   // SELL or stencil order
     if (bf16) {
       val[l] = nullptr;
       val16[l] = ar.alloc<__nv_bfloat16>(nv);
@@ -247,8 +247,9 @@ TailDesc<T> *MGHier<T>::make_tail(Arena &ar, const std::vector<MultiPtr<T>> &X, 
 }
 
 template <typename T>
-long MGHier<T>::sell_values(int l) const {
+long MGHier<T>::sell_values(int l, size_t value_size) const {
   if (kind == 2) return 9L * bpat[l]->sell.nent;
+  if (stencil(l, value_size)) return p2_values_count(p2lev[l]->n);
   return (kind == 0 ? 1L : 4L) * pat[l]->sell.nent;
 }
 
@@ -256,6 +257,8 @@ template <typename T>
 template <typename VT>
 void MGHier<T>::gather_values(int l, VT *out, cudaStream_t s) const {
   if (kind == 2) sell_gather9<VT>(bpat[l]->sell.nent, bmap[l], val64[l], out, s);
+  else if (stencil(l, sizeof(VT)))
+    p2_values<VT>(*p2lev[l], open_top, val64[l], false, out, l == 0 && sizeof(VT) < 8 ? copy64 : nullptr, s);
   else sell_gather<VT>(pat[l]->sell, kind == 0 ? 1 : 4, val64[l], out, s);
 }
 
@@ -264,7 +267,7 @@ void MGHier<T>::setup(cudaStream_t s) {
   for (int l = 0; l < nl; ++l) {
     if (bf16) gather_values<__nv_bfloat16>(l, val16[l], s);
     else gather_values<T>(l, val[l], s);
-    if (l == 0 && val0_64) gather_values<double>(0, val0_64, s);
+    if (l == 0 && val0_64 && val0_64 != copy64) gather_values<double>(0, val0_64, s);
     if (l == nl - 1 && !coarse_iter) break;
     if (kind == 1)
       jacobi_bsr2<T>(*pat[l], val64[l], diag[l], dinv[l], hi[l], partial, s);
@@ -287,21 +290,33 @@ void MGHier<T>::setup(cudaStream_t s) {
 }
 
 template <typename T>
-void MGHier<T>::op(int l, const T *u, T *out, SpmvMode mode, const SpmvArgs &a, cudaStream_t s) {
+void MGHier<T>::op(int l, const T *u, T *out, SpmvMode mode, const SpmvArgs &a, cudaStream_t s, P2Start start) {
   const int k = kind == 0 ? Profiler::P1_SPMV_L0 : Profiler::VEL_SPMV_L0;
   const bool timed = prof && l == 0;
   const int tk = timed ? prof->start(k, s) : -1;
-  spmv_level(l, u, out, mode, a, s);
+  spmv_level(l, u, out, mode, a, s, start);
   if (timed)
     prof->stop(k, tk, s,
                kind == 2 ? spmv_bytes(bpat[l]->nrows, bpat[l]->nnz, 9, n[l], bf16 ? 2 : sizeof(T), sizeof(T), mode,
                                       a.w != nullptr, false)
-                         : spmv_bytes(pat[l]->nrows, pat[l]->nnz, kind == 0 ? 1 : 4, n[l], bf16 ? 2 : sizeof(T),
-                                      sizeof(T), mode, a.w != nullptr, pat[l]->sell.stencil != 0));
+                         : spmv_bytes(pat[l]->nrows, pat[l]->nnz, kind == 0 ? 1 : stencil(l) ? 2 : 4, n[l],
+                                      bf16 ? 2 : sizeof(T), sizeof(T), mode, a.w != nullptr && start == P2_PLAIN,
+                                      pat[l]->sell.stencil != 0 || stencil(l)));
 }
 
 template <typename T>
-void MGHier<T>::spmv_level(int l, const T *u, T *out, SpmvMode mode, const SpmvArgs &a, cudaStream_t s) {
+void MGHier<T>::spmv_level(int l, const T *u, T *out, SpmvMode mode, const SpmvArgs &a, cudaStream_t s,
+                           P2Start start) {
+  if (stencil(l)) {
+    if constexpr (std::is_same<T, float>::value) {
+      if (bf16) {
+        p2_spmv<float, __nv_bfloat16>(*p2lev[l], open_top, p2tab[l], val16[l], u, out, mode, a, start, coef[l], s);
+        return;
+      }
+    }
+    p2_spmv<T, T>(*p2lev[l], open_top, p2tab[l], val[l], u, out, mode, a, start, coef[l], s);
+    return;
+  }
   if constexpr (std::is_same<T, float>::value) {
     if (bf16) {
       if (kind == 0) spmv_sell(*pat[l], val16[l], 1, u, out, mode, a, s);
@@ -356,11 +371,15 @@ void MGHier<T>::vcycle(int l, cudaStream_t s) {
   const int deg = l == nl - 1 ? kCoarseDegree : degree;
   T *cur = (deg - 1) % 2 == 0 ? x[l] : t[l];
   T *oth = cur == x[l] ? t[l] : x[l];
-  vec_scale_dinv<T>((int)n[l], coef[l], dinv[l], b[l], cur, s);
+  // the P2 stencil forms x_1 on the fly in the two sweeps that read it (in
+  // FP32: one launch and two vector streams less; FP64 sweeps are bound by
+  // their arithmetic, which forming x_1 at every neighbour would double)
+  const bool on_the_fly = stencil(l) && deg > 1 && sizeof(T) == 4;
+  if (!on_the_fly) vec_scale_dinv<T>((int)n[l], coef[l], dinv[l], b[l], cur, s);
   for (int k = 1; k < deg; ++k) {
     a.coef = coef[l] + 4 + 3 * (k - 1);
     a.w = k == 1 ? nullptr : oth;
-    op(l, cur, oth, SPMV_CHEB, a, s);
+    op(l, cur, oth, SPMV_CHEB, a, s, !on_the_fly || k > 2 ? P2_PLAIN : k == 1 ? P2_FIRST : P2_SECOND);
     std::swap(cur, oth);
   }
   if (l == nl - 1) return;
@@ -455,7 +474,7 @@ void MGHier<T>::enable_inner(Arena &ar, double rtol, int maxit, cudaStream_t bod
   acc = ar.alloc<double>(n[0]);
   if (!std::is_same<T, double>::value) {
     r64 = ar.alloc<double>(n[0]);
-    val0_64 = ar.alloc<double>(sell_values(0));
+    val0_64 = copy64 ? copy64 : ar.alloc<double>(sell_values(0, sizeof(double)));
   }
   ictl = ar.alloc<double>(8);
   iit = ar.alloc<int>(1);
@@ -497,6 +516,8 @@ void MGHier<T>::inner_residual(cudaStream_t s) {
     dot<double>(n[0], b[0], b[0], ictl + 1, ipartial, s);
   } else {
     if (kind == 0) spmv_sell<double>(*pat[0], val0_64, 1, acc, r64, SPMV_RES, a, s);
+    else if (stencil(0, sizeof(double)))
+      p2_spmv<double, double>(*p2lev[0], open_top, p2tab[0], val0_64, acc, r64, SPMV_RES, a, P2_PLAIN, nullptr, s);
     else if (kind == 1) spmv_sell_bsr2<double>(*pat[0], val0_64, acc, r64, SPMV_RES, a, s);
     else spmv_sell_bsr3<double>(*bpat[0], val0_64, acc, r64, SPMV_RES, a, s);
     dot<double>(n[0], r64, r64, ictl + 1, ipartial, s);

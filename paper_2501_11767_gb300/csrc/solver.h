@@ -5,6 +5,7 @@
 #include <mutex>
 
 #include "kernels.h"
+#include "p2stencil.h"
 
 namespace chnss {
 
@@ -71,6 +72,18 @@ struct MGHier {
   std::vector<const Transfer *> tr;
   std::vector<const Pattern *> bpat;   // kind 2: node patterns (3x3-block SELL) per level
   std::vector<const int *> bmap;       // kind 2: their map9 (value -> CSR position)
+  // kind 1 (set before init): mesh levels and stencil tables; a level that
+  // p2_applies() to is swept as a P2 stencil, any other one as 2x2-block SELL
+  std::vector<const Level *> p2lev;
+  std::vector<P2Table> p2tab;
+  int open_top = 0;
+  // level-0 values in FP64 and stencil order, written by setup with the
+  // level's own (T != double; null: not wanted)
+  double *copy64 = nullptr;
+  bool stencil(int l, size_t value_size) const {
+    return kind == 1 && !p2tab.empty() && p2_applies(*p2lev[l], p2tab[l], value_size);
+  }
+  bool stencil(int l) const { return stencil(l, sizeof(T)); }
   std::vector<long> n;
   int nc = 0;
   bool coarse_iter = false;   // coarsest level by Chebyshev steps (kCoarseDegree), no dense inverse
@@ -131,7 +144,8 @@ struct MGHier {
   TailDesc<T> *make_tail(Arena &ar, const std::vector<MultiPtr<T>> &X, const std::vector<MultiPtr<T>> &Tt,
                          const std::vector<MultiPtr<T>> &Rr, const std::vector<MultiPtr<T>> &B) const;
   // out = A_l u with the given epilogue (no profiling)
-  void spmv_level(int l, const T *u, T *out, SpmvMode mode, const SpmvArgs &a, cudaStream_t s);
+  void spmv_level(int l, const T *u, T *out, SpmvMode mode, const SpmvArgs &a, cudaStream_t s,
+                  P2Start start = P2_PLAIN);
 
  private:
   double *bsave = nullptr, *acc = nullptr;   // inner solve: right-hand side, iterate (FP64)
@@ -140,8 +154,8 @@ struct MGHier {
   double *ictl = nullptr, *ipartial = nullptr;
   int *iit = nullptr;
   cudaStream_t bodyq = nullptr;               // captures the WHILE body
-  void op(int l, const T *u, T *out, SpmvMode mode, const SpmvArgs &a, cudaStream_t s);
-  long sell_values(int l) const;                  // values of level l in SELL order
+  void op(int l, const T *u, T *out, SpmvMode mode, const SpmvArgs &a, cudaStream_t s, P2Start start = P2_PLAIN);
+  long sell_values(int l, size_t value_size) const;   // values of level l in SELL (or stencil) order
   template <typename VT>
   void gather_values(int l, VT *out, cudaStream_t s) const;   // FP64 CSR values -> SELL order
   void vcycle(int l, cudaStream_t s);
