@@ -142,6 +142,7 @@ struct Transfer {               // prolongation P (fine x coarse) and R = P^T
   double *Pv = nullptr, *Rv = nullptr;          // CSR order
   double *Ps = nullptr, *Rs = nullptr;          // SELL order
   float *Ps32 = nullptr, *Rs32 = nullptr;       // SELL order, FP32
+  int p1_cells = 0;                             // > 0: linear interpolation from a mesh of this many cells a side
 };
 
 struct Level {

@@ -220,6 +220,7 @@ namespace {
 // Linear interpolation of coarse P1 functions at the fine P1 nodes.
 void build_p1_transfer(Arena &ar, int nc, Transfer &t) {
   const int nf = 2 * nc, mf = nf + 1, mc = nc + 1;
+  t.p1_cells = nc;
   Pattern &P = t.P;
   P.nrows = mf * mf;
   P.ncols = mc * mc;

@@ -174,6 +174,14 @@ void MGHier<T>::init(Arena &ar, int kind_, bool singular_, const std::vector<con
   partial = partial_buf;
   sum = ar.alloc<double>(1);
   if (kind == 0 && !bf16) {
+    std::vector<MultiPtr<T>> X0(nl), B0(nl);
+    for (int l = 0; l < nl; ++l) {
+      X0[l].p[0] = x[l];
+      B0[l].p[0] = b[l];
+    }
+    mgc = mgc_plan<T>(ar, 1, pat, tr, val, dinv, coef, B0, X0, degree, coarse_iter, nc, cinv);
+  }
+  if (kind == 0 && !bf16 && mgc.first < 0) {
     for (int l = 1; l < nl; ++l)
       if (n[l] <= kTailRows) {
         tail_l0 = l;
@@ -341,6 +349,10 @@ static inline const T *transfer_vals(const Transfer &t, bool restrict_) {
 
 template <typename T>
 void MGHier<T>::vcycle(int l, cudaStream_t s) {
+  if (l == mgc.first) {
+    mgc_apply(mgc, s);
+    return;
+  }
   if (l == tail_l0) {
     mg_tail<T>(tail, 1, tail_width, s);
     return;
@@ -621,7 +633,10 @@ void MGBatch<T>::init(Arena &ar, MGHier<T> *hier, int nr_) {
       r[l].p[k] = ar.alloc<T>(h->n[l]);
       b[l].p[k] = ar.alloc<T>(h->n[l]);
     }
-  if (h->tail_l0 > 0) tail = h->make_tail(ar, x, t, r, b);
+  if (h->mgc.first >= 0)
+    mgc = mgc_plan<T>(ar, nr, h->pat, h->tr, h->val, h->dinv, h->coef, b, x, h->degree, h->coarse_iter, h->nc, h->cinv);
+  else if (h->tail_l0 > 0)
+    tail = h->make_tail(ar, x, t, r, b);
 }
 
 template <typename T>
@@ -646,6 +661,10 @@ void MGBatch<T>::op(int l, const MultiPtr<T> &u, const MultiPtr<T> &out, SpmvMod
 template <typename T>
 void MGBatch<T>::vcycle(int l, cudaStream_t s) {
   const int nl = h->nl;
+  if (l == mgc.first) {
+    mgc_apply(mgc, s);
+    return;
+  }
   if (l == h->tail_l0) {
     mg_tail<T>(tail, nr, h->tail_width, s);
     return;

@@ -5,6 +5,7 @@
 #include <mutex>
 
 #include "kernels.h"
+#include "mgcluster.h"
 #include "p2stencil.h"
 
 namespace chnss {
@@ -99,7 +100,10 @@ struct MGHier {
   std::vector<const double *> hi_ext;
   int degree = 2;          // Chebyshev smoothing degree (pre and post)
   double ratio = 4.0;      // smoothing interval [hi / ratio, hi]
-  // levels tail_l0.. (at most kTailRows rows each) run as one block launch
+  // coarse end in one launch: of a cluster on the structured meshes' P1
+  // levels (mgc.first..), otherwise of one block (tail_l0.., at most
+  // kTailRows rows each)
+  MgcPlan<T> mgc;
   int tail_l0 = -1;
   int tail_width = 8;            // widest tail row (operators and transfers): 8 or 16
   TailDesc<T> *tail = nullptr;   // device
@@ -175,6 +179,7 @@ struct MGBatch {
   int nr = 0;
   std::vector<MultiPtr<T>> x, t, r, b;     // per level
   TailDesc<T> *tail = nullptr;             // device, levels h->tail_l0..
+  MgcPlan<T> mgc;                          // or levels mgc.first.. by a cluster
   void init(Arena &ar, MGHier<T> *hier, int nr);
   T *input(int k) { return b[0].p[k]; }
   T *output(int k) { return x[0].p[k]; }
