@@ -34,7 +34,7 @@ void launch_cluster(void (*kernel)(P...), int ctas, int clusters, int threads, s
   at[0].val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  CHNSS_CK(cudaLaunchKernelEx(&cfg, kernel, P(args)...));
+  CHNSS_CK(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...));
 }
 
 }  // namespace chnss

@@ -14,6 +14,19 @@ namespace chnss {
 //   CHEB   out = c0 u + c1 w + c2 dinv (b - A u), (c0, c1, c2) = coef[0..2] (device)
 enum SpmvMode { SPMV_PLAIN = 0, SPMV_RES = 1, SPMV_ADD = 2, SPMV_CHEB = 3 };
 
+#ifdef __CUDACC__
+// Chebyshev step of one row, c0 u + c2 d (b - A u) (+ c1 w), with the roundings
+// of the per-sweep kernels written out: kernels that must give the same
+// iterates cannot leave the choice of fused multiply-adds to the compiler.
+__device__ __forceinline__ float fma_of(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_of(double a, double b, double c) { return fma(a, b, c); }
+template <typename T>
+__device__ __forceinline__ T cheb_step(T c0, T c1, T c2, T u, T d, T b, T au, bool has_w, T w) {
+  const T v = fma_of(c0, u, (c2 * d) * (b - au));
+  return has_w ? fma_of(c1, w, v) : v;
+}
+#endif
+
 // Up to kMaxRhs vectors that share one matrix (multi-right-hand-side kernels).
 constexpr int kMaxRhs = 3;
 template <typename T>

@@ -14,11 +14,76 @@ constexpr size_t kSmemLimit = 227 * 1024 - 1024;
 
 template <typename T> constexpr int mgc_threads() { return sizeof(T) == 4 ? 1024 : 512; }
 
+// owned lines [lb, le) of a level; entry (J, I) of a vector at base + J w + I
+struct Own {
+  int lb, le, base;
+};
 template <typename T>
-__device__ __forceinline__ T cheb(T c0, T c1, T c2, T ui, T di, T bi, T acc, bool has_w, T wi) {
-  T v = c0 * ui + c2 * di * (bi - acc);
-  if (has_w) v += c1 * wi;
-  return v;
+__device__ __forceinline__ Own own_lines(const MgcDesc<T> &d, int l, int me) {
+  const MgcLevel<T> &q = d.lv[l];
+  Own o;
+  o.lb = l < d.na ? q.lb[me] : 0;
+  o.le = l < d.na ? q.lb[me + 1] : q.w;
+  o.base = 1 - (o.lb - 1) * q.w;
+  return o;
+}
+
+// value v of owned row lr of the vector at `off` is also the halo of the
+// block below / above
+template <typename T>
+__device__ __forceinline__ void push(const MgcLevel<T> &q, const Own &o, T *sm, int off, int lr, T v) {
+  cg::cluster_group cl = cg::this_cluster();
+  const int me = (int)cl.block_rank();
+  if (lr < q.w && me > 0) {
+    const int below = o.lb - q.lb[me - 1];
+    *cl.map_shared_rank(sm + off + 1 + (below + 1) * q.w + lr, me - 1) = v;
+  }
+  const int last = (o.le - o.lb - 1) * q.w;
+  if (lr >= last && me + 1 < (int)cl.num_blocks()) *cl.map_shared_rank(sm + off + 1 + (lr - last), me + 1) = v;
+}
+
+// One sweep of the owned rows; cf null: b - A u, else a Chebyshev step.
+// where: 0 nothing more, 1 halo push, 2 gather in block 0's residual,
+// 3 result to global memory.
+template <typename T, int NR>
+__device__ __forceinline__ void sweep(const MgcDesc<T> &d, T *sm, int l, int u_off, int out_off, const double *cf,
+                                      bool has_w, int where) {
+  cg::cluster_group cl = cg::this_cluster();
+  const MgcLevel<T> &q = d.lv[l];
+  const Own o = own_lines(d, l, (int)cl.block_rank());
+  const int rows = (o.le - o.lb) * q.w, w = q.w;
+  T c0 = 0, c1 = 0, c2 = 0;
+  if (cf) {
+    c0 = (T)cf[0];
+    c1 = (T)cf[1];
+    c2 = (T)cf[2];
+  }
+  for (int lr = threadIdx.x; lr < rows; lr += blockDim.x) {
+    T v[7];
+#pragma unroll
+    for (int j = 0; j < 7; ++j) v[j] = sm[q.val_off + j * q.vs + lr];
+    const int e = 1 + w + lr;
+    const T di = sm[q.dinv_off + e];
+#pragma unroll
+    for (int k = 0; k < NR; ++k) {
+      const T *u = sm + u_off + k * q.vec + e;
+      const T ui = u[0];
+      T acc = v[0] * u[-w - 1];
+      acc = fma_of(v[1], u[-w], acc);
+      acc = fma_of(v[2], u[-1], acc);
+      acc = fma_of(v[3], ui, acc);
+      acc = fma_of(v[4], u[1], acc);
+      acc = fma_of(v[5], u[w], acc);
+      acc = fma_of(v[6], u[w + 1], acc);
+      const T bi = sm[q.b_off + k * q.vec + e];
+      T *out = sm + out_off + k * q.vec + e;
+      const T r = !cf ? bi - acc : cheb_step<T>(c0, c1, c2, ui, di, bi, acc, has_w, has_w ? *out : (T)0);
+      *out = r;
+      if (where == 1) push<T>(q, o, sm, out_off + k * q.vec, lr, r);
+      else if (where == 2) *cl.map_shared_rank(sm + d.r_off + k * d.r_vec + 1 + w + o.lb * w + lr, 0) = r;
+      else if (where == 3) d.x.p[k][o.lb * w + lr] = r;
+    }
+  }
 }
 
 // A V-cycle's levels from at most 128 (FP32) or 64 (FP64) cells a side down,
@@ -46,23 +111,14 @@ template <typename T, int NR>
 __global__ void __launch_bounds__(mgc_threads<T>()) k_p1_cluster(const MgcDesc<T> *__restrict__ dp) {
   extern __shared__ __align__(16) unsigned char raw[];
   T *sm = reinterpret_cast<T *>(raw);
-  __shared__ MgcDesc<T> d;
+  __shared__ __align__(16) unsigned char fixed[sizeof(MgcDesc<T>)];
+  MgcDesc<T> &d = *reinterpret_cast<MgcDesc<T> *>(fixed);
   cg::cluster_group cl = cg::this_cluster();
   const int me = (int)cl.block_rank(), ctas = (int)cl.num_blocks(), tid = threadIdx.x, nt = blockDim.x;
   for (int i = tid; i < (int)(sizeof(d) / 4); i += nt) reinterpret_cast<int *>(&d)[i] = reinterpret_cast<const int *>(dp)[i];
   __syncthreads();
 
-  struct Own {
-    int lb, le, base;   // owned lines [lb, le); entry (J, I) at base + J w + I
-  };
-  auto own = [&](int l) {
-    Own o;
-    const MgcLevel<T> &q = d.lv[l];
-    o.lb = l < d.na ? q.lb[me] : 0;
-    o.le = l < d.na ? q.lb[me + 1] : q.w;
-    o.base = 1 - (o.lb - 1) * q.w;
-    return o;
-  };
+  auto own = [&](int l) { return own_lines(d, l, me); };
   // load: values of the owned rows, Jacobi data with the halo, zeroed vectors
   for (int l = 0; l < d.nlev; ++l) {
     if (l >= d.na && me != 0) break;
@@ -94,56 +150,6 @@ __global__ void __launch_bounds__(mgc_threads<T>()) k_p1_cluster(const MgcDesc<T
     for (int e = tid; e < NR * d.lv[d.na].vec; e += nt) sm[d.lv[d.na].x_off + e] = 0;
   cl.sync();
 
-  // v at level l's own row lr of vector offset `off` is also the halo of the
-  // block below / above
-  auto push = [&](const MgcLevel<T> &q, const Own &o, int off, int lr, T v) {
-    if (lr < q.w && me > 0) {
-      const int below = o.lb - q.lb[me - 1];
-      *cl.map_shared_rank(sm + off + 1 + (below + 1) * q.w + lr, me - 1) = v;
-    }
-    const int last = (o.le - o.lb - 1) * q.w;
-    if (lr >= last && me + 1 < ctas) *cl.map_shared_rank(sm + off + 1 + (lr - last), me + 1) = v;
-  };
-  // one sweep of the owned rows; mode 0: b - A u -> out, 1: Chebyshev step
-  // where: 0 nothing more, 1 halo push, 2 gather in block 0's residual, 3 result to global memory
-  auto sweep = [&](int l, int u_off, int out_off, int mode, const double *cf, bool has_w, int where) {
-    const MgcLevel<T> &q = d.lv[l];
-    const Own o = own(l);
-    const int rows = (o.le - o.lb) * q.w, w = q.w;
-    T c0 = 0, c1 = 0, c2 = 0;
-    if (mode == 1) {
-      c0 = (T)cf[0];
-      c1 = (T)cf[1];
-      c2 = (T)cf[2];
-    }
-    for (int lr = tid; lr < rows; lr += nt) {
-      T v[7];
-#pragma unroll
-      for (int j = 0; j < 7; ++j) v[j] = sm[q.val_off + j * q.vs + lr];
-      const int e = 1 + w + lr;
-      const T di = sm[q.dinv_off + e];
-#pragma unroll
-      for (int k = 0; k < NR; ++k) {
-        const T *u = sm + u_off + k * q.vec + e;
-        T acc = 0;
-        acc += v[0] * u[-w - 1];
-        acc += v[1] * u[-w];
-        acc += v[2] * u[-1];
-        const T ui = u[0];
-        acc += v[3] * ui;
-        acc += v[4] * u[1];
-        acc += v[5] * u[w];
-        acc += v[6] * u[w + 1];
-        const T bi = sm[q.b_off + k * q.vec + e];
-        T *out = sm + out_off + k * q.vec + e;
-        const T r = mode == 0 ? bi - acc : cheb<T>(c0, c1, c2, ui, di, bi, acc, has_w, has_w ? *out : (T)0);
-        *out = r;
-        if (where == 1) push(q, o, out_off + k * q.vec, lr, r);
-        else if (where == 2) *cl.map_shared_rank(sm + d.r_off + k * d.r_vec + 1 + w + o.lb * w + lr, 0) = r;
-        else if (where == 3) d.x.p[k][o.lb * w + lr] = r;
-      }
-    }
-  };
   auto sync = [&](bool spread) {
     if (spread) cl.sync();
     else __syncthreads();
@@ -162,7 +168,7 @@ __global__ void __launch_bounds__(mgc_threads<T>()) k_p1_cluster(const MgcDesc<T
         sm[cur + k * q.vec + e] = c * sm[q.dinv_off + e] * sm[q.b_off + k * q.vec + e];
     __syncthreads();
     for (int s = 1; s < deg; ++s) {
-      sweep(l, cur, oth, 1, q.coef + 4 + 3 * (s - 1), s > 1, spread ? 1 : 0);
+      sweep<T, NR>(d, sm, l, cur, oth, q.coef + 4 + 3 * (s - 1), s > 1, spread ? 1 : 0);
       sync(spread);
       const int t = cur;
       cur = oth;
@@ -190,7 +196,7 @@ __global__ void __launch_bounds__(mgc_threads<T>()) k_p1_cluster(const MgcDesc<T
         acc += (T)0.5 * r[w];
         if (right) acc += (T)0.5 * r[w + 1];
         sm[q.b_off + k * q.vec + 1 + wc + lr] = acc;
-        if (spread) push(q, o, q.b_off + k * q.vec, lr, acc);
+        if (spread) push<T>(q, o, sm, q.b_off + k * q.vec, lr, acc);
       }
     }
   };
@@ -226,7 +232,7 @@ __global__ void __launch_bounds__(mgc_threads<T>()) k_p1_cluster(const MgcDesc<T
     int cur = q.x_off, oth = q.t_off;
     for (int s = 0; s < d.degree; ++s) {
       const bool last = s + 1 == d.degree;
-      sweep(l, cur, oth, 1, s == 0 ? q.coef + 1 : q.coef + 4 + 3 * (s - 1), s > 0, last && l == 0 ? 3 : spread ? 1 : 0);
+      sweep<T, NR>(d, sm, l, cur, oth, s == 0 ? q.coef + 1 : q.coef + 4 + 3 * (s - 1), s > 0, last && l == 0 ? 3 : spread ? 1 : 0);
       if (!(last && l == 0)) sync(spread);
       const int t = cur;
       cur = oth;
@@ -242,7 +248,7 @@ __global__ void __launch_bounds__(mgc_threads<T>()) k_p1_cluster(const MgcDesc<T
     from_zero(l, l == L ? d.coarse_degree : d.degree);
     if (l == L) break;
     const bool next = l + 1 < d.na;
-    sweep(l, q.x_off, q.t_off, 0, nullptr, false, next ? 1 : 2);
+    sweep<T, NR>(d, sm, l, q.x_off, q.t_off, nullptr, false, next ? 1 : 2);
     cl.sync();
     if (next) {
       restrict_to(l, q.t_off, q.vec, o.base, true);
@@ -282,7 +288,7 @@ __global__ void __launch_bounds__(mgc_threads<T>()) k_p1_cluster(const MgcDesc<T
       }
       if (l < L) {
         from_zero(l, d.degree);
-        sweep(l, q.x_off, q.t_off, 0, nullptr, false, 0);
+        sweep<T, NR>(d, sm, l, q.x_off, q.t_off, nullptr, false, 0);
         __syncthreads();
       } else if (d.coarse_degree > 0) {
         from_zero(l, d.coarse_degree);

@@ -1,31 +1,13 @@
 // P2 velocity stencil kernels (see p2stencil.h).
-#include "p2stencil.h"
+#include "p2slots.h"
 
 namespace chnss {
 namespace {
 
 constexpr int TPB = 256;
 
-// couplings of the four node types, in CSR (ascending lattice) order
-__host__ __device__ constexpr int slot_base(int ty) { return ty == 0 ? 0 : 10 + 9 * ty; }
-__host__ __device__ constexpr int slot_count(int ty) { return ty == 0 ? 19 : 9; }
-struct SlotTable {
-  signed char di[kP2Slots], dj[kP2Slots];
-};
-__host__ __device__ constexpr SlotTable slot_table() {
-  return {{-2, -1, 0, -2, -1, 0, 1, -2, -1, 0, 1, 2, -1, 0, 1, 2, 0, 1, 2,   // vertex
-           -1, -1, 0, -1, 0, 1, 0, 1, 1,                                     // horizontal edge
-           -2, -1, 0, -1, 0, 1, 0, 1, 2,                                     // vertical edge
-           -1, 0, 1, -1, 0, 1, -1, 0, 1},                                    // diagonal edge
-          {-2, -2, -2, -1, -1, -1, -1, 0, 0, 0, 0, 0, 1, 1, 1, 1, 2, 2, 2,
-           -2, -1, -1, 0, 0, 0, 1, 1, 2,
-           -1, -1, -1, 0, 0, 0, 1, 1, 1,
-           -1, -1, -1, 0, 0, 0, 1, 1, 1}};
-}
 constexpr SlotTable kSlots = slot_table();
 
-// type of the node at lattice parity (pi, pj)
-__host__ __device__ constexpr int type_of(int pi, int pj) { return (pi & 1) + 2 * (pj & 1); }
 // slot of the row of slot k's column that points back (its transposed entry)
 constexpr int back_slot(int ty, int k) {
   const int di = kSlots.di[slot_base(ty) + k], dj = kSlots.dj[slot_base(ty) + k];
@@ -54,10 +36,6 @@ static_assert(back_complete(), "the stencil is structurally symmetric");
 __constant__ SlotTable c_slots = kSlots;
 __constant__ BackTable c_back = kBack;
 
-__device__ __forceinline__ bool prescribed(int I, int J, int m, int open) {
-  return I <= 0 || J <= 0 || I >= m - 1 || (open ? J >= m : J >= m - 1);
-}
-
 template <typename T> struct V2;
 template <> struct V2<float> { using type = float2; };
 template <> struct V2<double> { using type = double2; };
@@ -73,8 +51,6 @@ __device__ __forceinline__ double2 load_pair(const double *p) { return __ldg(rei
 __device__ __forceinline__ float2 load_pair(const __nv_bfloat16 *p) {
   return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p));
 }
-__device__ __forceinline__ float fma_t(float a, float b, float c) { return fmaf(a, b, c); }
-__device__ __forceinline__ double fma_t(double a, double b, double c) { return fma(a, b, c); }
 template <typename T> __device__ __forceinline__ T from_double(double x) { return (T)x; }
 template <> __device__ __forceinline__ __nv_bfloat16 from_double<__nv_bfloat16>(double x) { return __double2bfloat16(x); }
 
@@ -114,13 +90,8 @@ struct NodeIn {
     if (mode == SPMV_PLAIN) return mk<T>(s0, s1);
     if (mode == SPMV_RES) return mk<T>(b.x - s0, b.y - s1);
     if (mode == SPMV_ADD) return mk<T>(b.x + s0, b.y + s1);
-    T v0 = c0 * ui.x + c2 * d.x * (b.x - s0);
-    T v1 = c0 * ui.y + c2 * d.y * (b.y - s1);
-    if (has_w) {
-      v0 += c1 * w.x;
-      v1 += c1 * w.y;
-    }
-    return mk<T>(v0, v1);
+    return mk<T>(cheb_step<T>(c0, c1, c2, ui.x, d.x, b.x, s0, has_w, w.x),
+                 cheb_step<T>(c0, c1, c2, ui.y, d.y, b.y, s1, has_w, w.y));
   }
 };
 
@@ -178,8 +149,8 @@ __global__ void __launch_bounds__(kSellMaxBlock, sizeof(T) == 4 ? 2 : 1) k_p2_sp
         const P v = load_pair(val + 2 * ((base + k) * ld + cell));
         const P xk = x[xi];
         if (di == oi && dj == oj) ui = xk;
-        s0 = fma_t(cf.c[2 * (top + base + k)], xk.y, fma_t((T)v.x, xk.x, s0));
-        s1 = fma_t((T)v.y, xk.y, fma_t(cf.c[2 * (top + base + k) + 1], xk.x, s1));
+        s0 = fma_of(cf.c[2 * (top + base + k)], xk.y, fma_of((T)v.x, xk.x, s0));
+        s1 = fma_of((T)v.y, xk.y, fma_of(cf.c[2 * (top + base + k) + 1], xk.x, s1));
       }
     }
     NodeIn<T> in;
@@ -398,8 +369,6 @@ void launch(const Level &L, int ks, const VT *val, const T *u, T *out, SpmvMode 
       case 4: k_p2_split<VT, 4, OPEN><<<gs, 128, 0, s>>>(L.n, ld, val, u, out, mode, start, a, tab); return;
       case 8: k_p2_split<VT, 8, OPEN><<<gs, 256, 0, s>>>(L.n, ld, val, u, out, mode, start, a, tab); return;
     }
-  } else if (ks != 1) {
-    throw Error{CHNSS_ERR_ARG, "FP64 velocity stencil: fine levels only"};
   }
   k_p2_spmv<T, VT, OPEN, true><<<nb, tpb, 0, s>>>(L.n, ld, val, u, out, mode, start, a, cf);
 }
@@ -412,6 +381,95 @@ double rounded(double x, const double *) { return x; }
 float rounded(double x, const float *) { return (float)x; }
 float rounded(double x, const __nv_bfloat16 *) { return __bfloat162float(__double2bfloat16(x)); }
 }  // namespace
+
+namespace {
+__constant__ P2Transfers c_transfers = p2_transfers();
+
+// Grid transfers of the velocity with their columns and weights computed:
+// the SELL form streamed 8 bytes an entry (10.7 entries a fine node, both
+// ways) beside the vectors.  Entries in CSR order, so results are the same
+// bit for bit.  One thread a coarse node of the type (blockIdx.z the parity
+// of I, so that a warp's nodes share a type).
+template <typename T, bool OPEN>
+__global__ void k_p2_restrict(int nc, const T *__restrict__ r, T *__restrict__ b) {
+  using P = typename V2<T>::type;
+  constexpr int open = OPEN ? 1 : 0;
+  const int mc = 2 * nc + 1, m = 4 * nc + 1;
+  const int I = 2 * (blockIdx.x * blockDim.x + threadIdx.x) + blockIdx.z, J = blockIdx.y;
+  if (I >= mc) return;
+  T a0 = 0, a1 = 0;
+  if (!prescribed(I, J, mc, open)) {
+    const P *r2 = reinterpret_cast<const P *>(r) + (long)(2 * J) * m + 2 * I;
+    auto sum = [&](auto tyc) {
+      constexpr P2Transfers t = p2_transfers();
+      constexpr int ty = decltype(tyc)::value, cnt = t.rn[ty];
+#pragma unroll
+      for (int k = 0; k < cnt; ++k) {
+        P x = mk<T>(0, 0);
+        if (!OPEN || 2 * J + t.rj[ty][k] < m) x = r2[t.rj[ty][k] * m + t.ri[ty][k]];   // else above the top
+        a0 = fma_of((T)t.rw[ty][k], x.x, a0);
+        a1 = fma_of((T)t.rw[ty][k], x.y, a1);
+      }
+    };
+    switch (type_of(I, J)) {
+      case 0: sum(std::integral_constant<int, 0>()); break;
+      case 1: sum(std::integral_constant<int, 1>()); break;
+      case 2: sum(std::integral_constant<int, 2>()); break;
+      default: sum(std::integral_constant<int, 3>());
+    }
+  }
+  reinterpret_cast<P *>(b)[(long)J * mc + I] = mk<T>(a0, a1);
+}
+
+// x += P xc, one thread a fine node
+template <typename T>
+__global__ void k_p2_prolong(int nc, int open, const T *__restrict__ xc, T *__restrict__ x) {
+  using P = typename V2<T>::type;
+  __shared__ float w[4][6];
+  __shared__ int off[4][6], cnt[4];
+  const int mc = 2 * nc + 1, m = 4 * nc + 1, J = blockIdx.y;
+  if (threadIdx.x < 24) {   // the line's four classes
+    const int c = 4 * (J & 3) + threadIdx.x / 6, k = threadIdx.x % 6;
+    w[threadIdx.x / 6][k] = c_transfers.pw[c][k];
+    off[threadIdx.x / 6][k] = c_transfers.pj[c][k] * mc + c_transfers.pi[c][k];
+    if (k == 0) cnt[threadIdx.x / 6] = c_transfers.pn[c];
+  }
+  __syncthreads();
+  const int I = blockIdx.x * blockDim.x + threadIdx.x;
+  if (prescribed(I, J, m, open)) return;
+  P *xi = reinterpret_cast<P *>(x) + (long)J * m + I;
+  const P *c = reinterpret_cast<const P *>(xc) + (long)(2 * (J >> 2)) * mc + 2 * (I >> 2);
+  const int q = I & 3, n = cnt[q];
+  const P old = *xi;
+  T a0 = 0, a1 = 0;
+#pragma unroll
+  for (int k = 0; k < 6; ++k)
+    if (k < n) {
+      const P v = c[off[q][k]];
+      a0 = fma_of((T)w[q][k], v.x, a0);
+      a1 = fma_of((T)w[q][k], v.y, a1);
+    }
+  *xi = mk<T>(old.x + a0, old.y + a1);
+}
+}  // namespace
+
+template <typename T>
+void p2_restrict(int nc, int open_top, const T *r, T *b, cudaStream_t s) {
+  const dim3 g((unsigned)((nc + 1 + 127) / 128), (unsigned)(2 * nc + 1), 2);
+  if (open_top) k_p2_restrict<T, true><<<g, 128, 0, s>>>(nc, r, b);
+  else k_p2_restrict<T, false><<<g, 128, 0, s>>>(nc, r, b);
+  CHNSS_LAUNCH_CK();
+}
+template <typename T>
+void p2_prolong_add(int nc, int open_top, const T *xc, T *x, cudaStream_t s) {
+  const dim3 g((unsigned)((4 * nc + 1 + 255) / 256), (unsigned)(4 * nc + 1));
+  k_p2_prolong<T><<<g, 256, 0, s>>>(nc, open_top, xc, x);
+  CHNSS_LAUNCH_CK();
+}
+template void p2_restrict<float>(int, int, const float *, float *, cudaStream_t);
+template void p2_restrict<double>(int, int, const double *, double *, cudaStream_t);
+template void p2_prolong_add<float>(int, int, const float *, float *, cudaStream_t);
+template void p2_prolong_add<double>(int, int, const double *, double *, cudaStream_t);
 
 template <typename T, typename VT>
 void p2_spmv(const Level &L, int open_top, const P2Table &tab, const VT *val, const T *u, T *out, SpmvMode mode,

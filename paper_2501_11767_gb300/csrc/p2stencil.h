@@ -59,4 +59,11 @@ template <typename T, typename VT>
 void p2_spmv(const Level &L, int open_top, const P2Table &tab, const VT *val, const T *u, T *out, SpmvMode mode,
              const SpmvArgs &a, P2Start start, const double *scale, cudaStream_t s);
 
+// b = R r onto the mesh of nc cells a side; x += P xc from it (velocity
+// transfers of build_vel_transfer, the same sums; vectors aligned to a node)
+template <typename T>
+void p2_restrict(int nc, int open_top, const T *r, T *b, cudaStream_t s);
+template <typename T>
+void p2_prolong_add(int nc, int open_top, const T *xc, T *x, cudaStream_t s);
+
 }  // namespace chnss

@@ -401,12 +401,15 @@ void MGHier<T>::vcycle(int l, cudaStream_t s) {
   op(l, x[l], r[l], SPMV_RES, ar, s);
   const Transfer &T_ = *tr[l];
   SpmvArgs none;
-  spmv_sell<T>(T_.R, transfer_vals<T>(T_, true), nc_, r[l], b[l + 1], SPMV_PLAIN, none, s);
+  const bool p2 = kind == 1 && !p2lev.empty();   // structured velocity transfers
+  if (p2) p2_restrict<T>(p2lev[l + 1]->n, open_top, r[l], b[l + 1], s);
+  else spmv_sell<T>(T_.R, transfer_vals<T>(T_, true), nc_, r[l], b[l + 1], SPMV_PLAIN, none, s);
   const int kc = kind == 0 ? Profiler::P1_MG_COARSE : Profiler::VEL_MG_COARSE;
   const int tkc = prof && l == 0 ? prof->start(kc, s) : -1;
   vcycle(l + 1, s);
   if (prof && l == 0) prof->stop(kc, tkc, s, 0.0);   // time only: every level below the finest
-  spmv_sell<T>(T_.P, transfer_vals<T>(T_, false), nc_, x[l + 1], x[l], SPMV_ADD, none, s);
+  if (p2) p2_prolong_add<T>(p2lev[l + 1]->n, open_top, x[l + 1], x[l], s);
+  else spmv_sell<T>(T_.P, transfer_vals<T>(T_, false), nc_, x[l + 1], x[l], SPMV_ADD, none, s);
   // post-smoothing from x_0 = x[l]
   a.coef = coef[l] + 1;
   a.w = nullptr;
