@@ -588,6 +588,8 @@ void init_precset(chnss_ctx *c, PrecSet<T> &P) {
   for (int l = 0; l < nl; ++l) P.A.p2lev.push_back(&c->lv(l));
   P.A.p2tab = c->p2tab;
   P.A.open_top = c->mesh->m.top_bc;
+  P.A.degree = 4;        // velocity smoothing: degree 4 on [hi / 16, hi]
+  P.A.ratio = 16.0;
   P.A.init(ar, 1, false, p2s, d2s, vals(c->A), tvs, c->partial);
   // the fine operator applied inside FGMRES: in stencil order it is the FP64
   // hierarchy's own level 0, or a copy written together with the FP32 values
@@ -597,8 +599,6 @@ void init_precset(chnss_ctx *c, PrecSet<T> &P) {
     c->As = P.A.copy64 = ar.alloc<double>(p2_values_count(c->lv(0).n));
   else
     c->As = ar.alloc<double>(4L * c->lv(0).p2.sell.nent);
-  P.A.degree = 4;        // velocity smoothing: degree 4 on [hi / 16, hi]
-  P.A.ratio = 16.0;
   P.Kp.keep_dense = true;       // a pure Laplacian: its coarsest level is not mass-dominated
   if (c->mesh->m.top_bc == 1)   // open top: Dirichlet outflow rows, non-singular
     P.Kp.init(ar, 0, false, p1s, d1s, vals(c->Kpd), t1s, c->partial);

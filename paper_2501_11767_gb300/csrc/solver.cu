@@ -136,6 +136,8 @@ void MGHier<T>::init(Arena &ar, int kind_, bool singular_, const std::vector<con
   if (bf16 && !std::is_same<T, float>::value) throw Error{CHNSS_ERR_ARG, "BF16 values need FP32 vectors"};
   if (kind == 2 && ((int)bpat.size() != nl || (int)bmap.size() != nl))
     throw Error{CHNSS_ERR_ARG, "3x3-block levels need a node pattern and value map per level"};
+  nc = (kind == 1 ? 2 : 1) * pat[nl - 1]->nrows;
+  coarse_iter = nl > 1 && !singular && !keep_dense && nc > kCoarseDenseMax;
   n.resize(nl);
   val.resize(nl);
   val16.assign(nl, nullptr);
@@ -164,8 +166,6 @@ void MGHier<T>::init(Arena &ar, int kind_, bool singular_, const std::vector<con
     hi[l] = ar.alloc<double>(1);
     coef[l] = ar.alloc<double>(4 + 3 * (kMaxSmoothDegree - 1));
   }
-  nc = (int)n[nl - 1];
-  coarse_iter = nl > 1 && !singular && !keep_dense && nc > kCoarseDenseMax;
   if (!coarse_iter) {
     dense = ar.alloc<double>((long)nc * nc);
     cinv = ar.alloc<double>((long)nc * nc);
@@ -173,6 +173,10 @@ void MGHier<T>::init(Arena &ar, int kind_, bool singular_, const std::vector<con
   status = ar.alloc<int>(1);
   partial = partial_buf;
   sum = ar.alloc<double>(1);
+  if constexpr (std::is_same<T, float>::value) {
+    if (kind == 1 && !p2tab.empty())
+      vlc = vlc_plan(ar, p2lev, open_top, p2tab, val, val16, dinv, coef, b, x, degree, coarse_iter, nc, cinv);
+  }
   if (kind == 0 && !bf16) {
     std::vector<MultiPtr<T>> X0(nl), B0(nl);
     for (int l = 0; l < nl; ++l) {
@@ -351,6 +355,10 @@ template <typename T>
 void MGHier<T>::vcycle(int l, cudaStream_t s) {
   if (l == mgc.first) {
     mgc_apply(mgc, s);
+    return;
+  }
+  if (l == vlc.first) {
+    vlc_apply(vlc, s);
     return;
   }
   if (l == tail_l0) {
