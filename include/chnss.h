@@ -478,7 +478,7 @@ chnss_status chnss3_objective(chnss3_ctx_t ctx, const double *phi_p, double *J, 
  * Every call shares the one array and overwrites it (the solver rewrites all
  * of it before reading), so calls whose work overlaps on the GPU (different
  * streams, threads or contexts at the same time) race and must not be
- * issued.  Synchronises ctx's stream once per iteration. */
+ * issued.  Synchronises ctx's stream once every eight iterations. */
 chnss_status chnss_mass_solve_noalloc(chnss_ctx_t ctx, const double *rhs, double *x_out,
                                       chnss_solve_info *info);
 

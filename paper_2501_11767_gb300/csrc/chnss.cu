@@ -1932,6 +1932,7 @@ chnss_status mass_solve_noalloc(chnss_ctx *c, const double *b, double *x, chnss_
   view.V = base + n;                     // z, p, q
   view.partial = base + 4L * kNoAllocMaxN1;
   view.sc = view.partial + kNoAllocPartials;
+  view.counter = reinterpret_cast<int *>(view.sc + 8);
   view.hstat = c->pinned + 12;
   return pcg(P, c->M1[0], c->dinvM, b, x, 1e-12, 1000, view, info, c->s);
 }

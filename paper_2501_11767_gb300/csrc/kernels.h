@@ -265,12 +265,21 @@ void hessenberg_solve_dev(const int *k, int ldh, const double *H, const double *
 void combine_columns_dev(long n, const double *Z, long ldz, const int *k, const double *y, double *x,
                          cudaStream_t s);
 void set_scalar(double *dst, const double *src, double scale, bool sqrt_first, cudaStream_t s);
-// PCG scalars: alpha = rz / pq
-void pcg_alpha(const double *rz, const double *pq, double *alpha, cudaStream_t s);
-void pcg_update_xr(long n, const double *alpha, const double *p, const double *q, double *x, double *r,
-                   cudaStream_t s);
-void pcg_update_p(long n, const double *rz_new, const double *rz_old, const double *z, double *p, cudaStream_t s);
-void vec_mul(long n, const double *a, const double *b, double *out, cudaStream_t s);
+// Jacobi PCG in two kernels an iteration, its decisions on the device.
+// Scalars of a solve (sc); done: PCG_RUNNING until a decision ends it, after
+// which further iterations do nothing.
+enum PcgScalar { PCG_RZ = 0, PCG_BETA, PCG_TARGET, PCG_ALPHA, PCG_BNORM, PCG_RNORM, PCG_ITERS, PCG_DONE };
+enum PcgDone { PCG_RUNNING = 0, PCG_CONVERGED, PCG_NAN, PCG_MAXIT };
+struct PcgWork {
+  double *r, *q, *sc, *partial;
+  int *counter;
+};
+// r = b, x = 0, p = 0, sc from them (x may alias b)
+void pcg_start(long n, const double *dinv, const double *b, double *x, double *p, double rtol, const PcgWork &w,
+               cudaStream_t s);
+// one iteration with the previous direction p_old (not read by the first); the new one goes to p_new
+void pcg_iteration(const Pattern &P, const double *val, const double *dinv, double *x, const double *p_old,
+                   double *p_new, int maxit, const PcgWork &w, cudaStream_t s);
 
 // dense coarse-grid inverse (one CTA, Gauss-Jordan with partial pivoting)
 void coarse_dense_csr(const Pattern &P, const double *val, double add_all, double *dense, cudaStream_t s);

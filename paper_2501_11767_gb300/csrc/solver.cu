@@ -756,6 +756,7 @@ void KrylovWork::init(Arena &ar, int m_, long nmax_, double *pinned, bool pairs)
   hstat = pinned;
   dv = ar.alloc<double>(8);
   di = ar.alloc<int>(8);
+  counter = ar.alloc<int>(1);
 }
 
 namespace {
@@ -1135,37 +1136,17 @@ __global__ void k_fg_cycle_end(const double *sc, double *dv, int *di, int maxit,
   }
   cudaGraphSetConditional(hw, more ? 1u : 0u);
 }
-// PCG: sc[0] = ||b||^2 (b copied to r)
-__global__ void k_pcg_init(const double *sc, double *dv, int *di, double rtol, cudaGraphConditionalHandle hw) {
-  const double bn = sqrt(sc[0]);
-  dv[0] = bn;
-  dv[1] = rtol * bn;
-  dv[2] = bn;
-  for (int i = 0; i < 8; ++i) di[i] = 0;
-  bool more = true;
-  if (!isfinite(bn)) {
-    di[2] = CHNSS_ERR_NAN;
-    more = false;
-  } else if (bn <= dv[1]) {
-    di[3] = 1;
-    more = false;
-  }
-  cudaGraphSetConditional(hw, more ? 1u : 0u);
+// the PCG's loop condition, and its outcome in the device-driven records
+__global__ void k_pcg_gate(const double *sc, double *dv, int *di, cudaGraphConditionalHandle hw) {
+  const int done = (int)sc[PCG_DONE];
+  dv[0] = sc[PCG_BNORM];
+  dv[1] = sc[PCG_TARGET];
+  dv[2] = sc[PCG_RNORM];
+  di[0] = (int)sc[PCG_ITERS];
+  di[2] = done == PCG_NAN ? CHNSS_ERR_NAN : done == PCG_MAXIT ? CHNSS_ERR_NOCONV : CHNSS_OK;
+  di[3] = done == PCG_CONVERGED;
+  cudaGraphSetConditional(hw, done == PCG_RUNNING ? 1u : 0u);
 }
-// after an iteration: sc[5] = ||r||^2
-__global__ void k_pcg_decide(const double *sc, double *dv, int *di, int maxit, cudaGraphConditionalHandle hw) {
-  const int it = di[0] + 1;
-  di[0] = it;
-  const double rn = sqrt(sc[5]);
-  dv[2] = rn;
-  bool more = false;
-  if (!isfinite(rn)) di[2] = CHNSS_ERR_NAN;
-  else if (rn <= dv[1]) di[3] = 1;
-  else if (it >= maxit) di[2] = CHNSS_ERR_NOCONV;
-  else more = true;
-  cudaGraphSetConditional(hw, more ? 1u : 0u);
-}
-__global__ void k_copy_scalar(const double *src, double *dst) { *dst = *src; }
 __global__ void k_krylov_record(const double *dv, const int *di, double *dst) {
   dst[0] = (double)di[0];
   dst[1] = (double)di[3];
@@ -1289,31 +1270,17 @@ void fgmres_record(LinearOperator &A, const double *b, double *x, double rtol, d
 void pcg_record(const Pattern &P, const double *val, const double *dinv, const double *b, double *x, double rtol,
                 int maxit, KrylovWork &ws, cudaStream_t s, cudaStream_t bq1) {
   const long n = P.nrows;
-  double *r = ws.w, *z = ws.V, *p = ws.V + n, *q = ws.V + 2 * n;
-  double *sc = ws.sc;   // [0] bb [1] rz [2] rz_new [3] pq [4] alpha [5] rr
-  vec_copy(n, b, r, s);
-  dot<double>(n, r, r, sc, ws.partial, s);
-  vec_fill(n, 0.0, x, s);
+  double *p0 = ws.V, *p1 = ws.V + n;
+  const PcgWork w = {ws.w, ws.V + 2 * n, ws.sc, ws.partial, ws.counter};
+  pcg_start(n, dinv, b, x, p1, rtol, w, s);
   const cudaGraphConditionalHandle hw = new_handle(s);
-  k_pcg_init<<<1, 1, 0, s>>>(sc, ws.dv, ws.di, rtol, hw);
+  k_pcg_gate<<<1, 1, 0, s>>>(ws.sc, ws.dv, ws.di, hw);
   CHNSS_LAUNCH_CK();
-  vec_mul(n, dinv, r, z, s);
-  vec_copy(n, z, p, s);
-  dot<double>(n, r, z, sc + 1, ws.partial, s);
+  // two iterations a body: the directions alternate between two vectors
   record_body(s, bq1, hw, cudaGraphCondTypeWhile, [&] {
-    SpmvArgs none;
-    spmv_csr<double>(P, val, 1, p, q, SPMV_PLAIN, none, bq1);
-    dot<double>(n, p, q, sc + 3, ws.partial, bq1);
-    pcg_alpha(sc + 1, sc + 3, sc + 4, bq1);
-    pcg_update_xr(n, sc + 4, p, q, x, r, bq1);
-    dot<double>(n, r, r, sc + 5, ws.partial, bq1);
-    k_pcg_decide<<<1, 1, 0, bq1>>>(sc, ws.dv, ws.di, maxit, hw);
-    CHNSS_LAUNCH_CK();
-    // the next direction (unused once the loop has stopped)
-    vec_mul(n, dinv, r, z, bq1);
-    dot<double>(n, r, z, sc + 2, ws.partial, bq1);
-    pcg_update_p(n, sc + 2, sc + 1, z, p, bq1);
-    k_copy_scalar<<<1, 1, 0, bq1>>>(sc + 2, sc + 1);
+    pcg_iteration(P, val, dinv, x, p1, p0, maxit, w, bq1);
+    pcg_iteration(P, val, dinv, x, p0, p1, maxit, w, bq1);
+    k_pcg_gate<<<1, 1, 0, bq1>>>(ws.sc, ws.dv, ws.di, hw);
     CHNSS_LAUNCH_CK();
   });
 }
@@ -1327,52 +1294,31 @@ chnss_status pcg(const Pattern &P, const double *val, const double *dinv, const 
                  int maxit, KrylovWork &ws, chnss_solve_info *info, cudaStream_t s) {
   const auto t0 = std::chrono::steady_clock::now();
   const long n = P.nrows;
-  double *r = ws.w, *z = ws.V, *p = ws.V + n, *q = ws.V + 2 * n;
-  double *sc = ws.sc;   // [0] bb [1] rz [2] rz_new [3] pq [4] alpha [5] rr
-  // b is read only here, into r, before x is cleared: x may alias b
-  vec_copy(n, b, r, s);
-  dot<double>(n, r, r, sc, ws.partial, s);
-  vec_fill(n, 0.0, x, s);
-  const double bnorm = std::sqrt(read_scalar(sc, ws.hstat, s));
-  const double target = rtol * bnorm;
-  double rn = bnorm;
-  int it = 0;
-  bool converged = false;
-  chnss_status st = CHNSS_OK;
-  if (!std::isfinite(bnorm)) {
-    st = CHNSS_ERR_NAN;
-  } else if (bnorm <= target) {
-    converged = true;
-  } else {
-    vec_mul(n, dinv, r, z, s);
-    vec_copy(n, z, p, s);
-    dot<double>(n, r, z, sc + 1, ws.partial, s);
-    double *rz = sc + 1, *rzn = sc + 2;
-    SpmvArgs none;
-    while (it < maxit) {
-      spmv_csr<double>(P, val, 1, p, q, SPMV_PLAIN, none, s);
-      dot<double>(n, p, q, sc + 3, ws.partial, s);
-      pcg_alpha(rz, sc + 3, sc + 4, s);
-      pcg_update_xr(n, sc + 4, p, q, x, r, s);
-      ++it;
-      dot<double>(n, r, r, sc + 5, ws.partial, s);
-      rn = std::sqrt(read_scalar(sc + 5, ws.hstat, s));
-      if (!std::isfinite(rn)) { st = CHNSS_ERR_NAN; break; }
-      if (rn <= target) { converged = true; break; }
-      vec_mul(n, dinv, r, z, s);
-      dot<double>(n, r, z, rzn, ws.partial, s);
-      pcg_update_p(n, rzn, rz, z, p, s);
-      std::swap(rz, rzn);
+  double *p0 = ws.V, *p1 = ws.V + n;
+  const PcgWork w = {ws.w, ws.V + 2 * n, ws.sc, ws.partial, ws.counter};
+  // b is read only here, element by element, before x is cleared: x may alias b
+  pcg_start(n, dinv, b, x, p1, rtol, w, s);
+  // the device decides when to stop; iterations queued past that do nothing,
+  // so the host looks only every kAhead of them
+  constexpr int kAhead = 8;
+  int done = PCG_RUNNING, queued = 0;
+  do {
+    for (int k = 0; k < kAhead && queued < maxit; ++k, ++queued) {
+      pcg_iteration(P, val, dinv, x, p1, p0, maxit, w, s);
+      std::swap(p0, p1);
     }
-    if (!converged && st == CHNSS_OK) st = CHNSS_ERR_NOCONV;
-  }
+    CHNSS_CK(cudaMemcpyAsync(ws.hstat, ws.sc + PCG_BNORM, 4 * sizeof(double), cudaMemcpyDeviceToHost, s));
+    CHNSS_CK(cudaStreamSynchronize(s));
+    done = (int)ws.hstat[PCG_DONE - PCG_BNORM];
+  } while (done == PCG_RUNNING && queued < maxit);
+  const double bnorm = ws.hstat[0], rn = ws.hstat[PCG_RNORM - PCG_BNORM];
   if (info) {
-    info->iters = it;
-    info->converged = converged ? 1 : 0;
+    info->iters = (int)ws.hstat[PCG_ITERS - PCG_BNORM];
+    info->converged = done == PCG_CONVERGED ? 1 : 0;
     info->rel_residual = bnorm > 0 ? rn / bnorm : 0.0;
     info->seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
   }
-  return st;
+  return done == PCG_CONVERGED ? CHNSS_OK : done == PCG_NAN ? CHNSS_ERR_NAN : CHNSS_ERR_NOCONV;
 }
 
 }  // namespace chnss

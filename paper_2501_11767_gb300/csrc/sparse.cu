@@ -872,11 +872,6 @@ __global__ void k_sub_mean(int n, T *x, const double *sum) {
   const int i = blockIdx.x * TPB + threadIdx.x;
   if (i < n) x[i] = (T)((double)x[i] - *sum / n);
 }
-__global__ void k_mul(long n, const double *a, const double *b, double *out) {
-  const long i = (long)blockIdx.x * TPB + threadIdx.x;
-  if (i < n) out[i] = a[i] * b[i];
-}
-
 // --------------------------------------------------------------------------
 // reductions
 __device__ __forceinline__ double block_sum(double v, double *sm) {
@@ -1019,18 +1014,119 @@ __global__ void k_set_scalar(double *dst, const double *src, double scale, int s
   const double v = sq ? sqrt(*src) : *src;
   *dst = scale * v;
 }
-__global__ void k_pcg_alpha(const double *rz, const double *pq, double *alpha) { *alpha = *rz / *pq; }
-__global__ void k_pcg_xr(long n, const double *alpha, const double *p, const double *q, double *x, double *r) {
-  const long i = (long)blockIdx.x * TPB + threadIdx.x;
-  if (i < n) {
-    const double a = *alpha;
-    x[i] += a * p[i];
-    r[i] -= a * q[i];
+
+// Jacobi PCG, two kernels an iteration: the direction p = z + beta p_old with
+// z = D^-1 r is formed where it is read (at every neighbour of a row, in
+// place of a pass of its own), the block that finishes last sums the partials
+// in order and takes the decisions.  One thread a row: the FP64 pipe bounds
+// the products (8 lanes a row, whose steps and shuffles all issue for every
+// lane: 37 us an iteration at 240^2; 65 as 11 launches and a host round trip).
+// Sum of v over the block, in thread 0.
+__device__ __forceinline__ double block_sum0(double v, double *sm) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x == 0)
+    for (int k = 0; k < TPB / 32; ++k) t += sm[k];
+  return t;
+}
+// Sums of NQ values v over the grid; true in the last block, out in its thread 0.
+template <int NQ>
+__device__ bool grid_sums(const double (&v)[NQ], double *partial, int *counter, double (&out)[NQ]) {
+  __shared__ double sm[TPB / 32];
+  __shared__ bool last;
+  const int nb = gridDim.x;
+  for (int q = 0; q < NQ; ++q) {
+    const double t = block_sum0(v[q], sm);
+    if (threadIdx.x == 0) partial[q * nb + blockIdx.x] = t;
+  }
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(counter, 1) == nb - 1;
+  }
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  for (int q = 0; q < NQ; ++q) {
+    double t = 0.0;
+    for (int b = threadIdx.x; b < nb; b += TPB) t += __ldcg(partial + q * nb + b);
+    out[q] = block_sum0(t, sm);
+  }
+  if (threadIdx.x == 0) *counter = 0;
+  return true;
+}
+
+__global__ void __launch_bounds__(TPB) k_pcg_start(long n, const double *dinv, const double *b, double *x, double *p,
+                                                   double rtol, PcgWork w) {
+  double v[2] = {0.0, 0.0}, t[2];
+  for (long i = (long)blockIdx.x * TPB + threadIdx.x; i < n; i += (long)gridDim.x * TPB) {
+    const double r = b[i];
+    w.r[i] = r;
+    x[i] = 0.0;
+    p[i] = 0.0;
+    v[0] += r * r;
+    v[1] += r * (dinv[i] * r);
+  }
+  if (grid_sums<2>(v, w.partial, w.counter, t) && threadIdx.x == 0) {
+    const double bn = sqrt(t[0]);
+    w.sc[PCG_RZ] = t[1];
+    w.sc[PCG_BETA] = 0.0;
+    w.sc[PCG_TARGET] = rtol * bn;
+    w.sc[PCG_BNORM] = w.sc[PCG_RNORM] = bn;
+    w.sc[PCG_ITERS] = 0.0;
+    w.sc[PCG_DONE] = !isfinite(bn) ? PCG_NAN : bn <= rtol * bn ? PCG_CONVERGED : PCG_RUNNING;
   }
 }
-__global__ void k_pcg_p(long n, const double *rzn, const double *rzo, const double *z, double *p) {
-  const long i = (long)blockIdx.x * TPB + threadIdx.x;
-  if (i < n) p[i] = z[i] + (*rzn / *rzo) * p[i];
+
+// p = z + beta p_old; q = A p; alpha = r.z / p.q
+__global__ void __launch_bounds__(TPB) k_pcg_apply(int nrows, const int *__restrict__ rowptr, const int *__restrict__ col,
+                                                   const double *__restrict__ val, const double *__restrict__ dinv,
+                                                   const double *__restrict__ p_old, double *__restrict__ p_new,
+                                                   PcgWork w) {
+  if (w.sc[PCG_DONE] != PCG_RUNNING) return;
+  const double beta = w.sc[PCG_BETA];
+  const double *__restrict__ r = w.r;
+  double v[1] = {0.0}, t[1];
+  for (int row = blockIdx.x * TPB + threadIdx.x; row < nrows; row += gridDim.x * TPB) {
+    const int k0 = rowptr[row], k1 = rowptr[row + 1];
+    double acc = 0.0;
+#pragma unroll 8
+    for (int k = k0; k < k1; ++k) {
+      const int c = col[k];
+      acc += val[k] * (dinv[c] * r[c] + beta * p_old[c]);
+    }
+    const double p = dinv[row] * r[row] + beta * p_old[row];
+    p_new[row] = p;
+    w.q[row] = acc;
+    v[0] += p * acc;
+  }
+  if (grid_sums<1>(v, w.partial, w.counter, t) && threadIdx.x == 0) w.sc[PCG_ALPHA] = w.sc[PCG_RZ] / t[0];
+}
+
+// x += alpha p, r -= alpha q, the norms and the next beta
+__global__ void __launch_bounds__(TPB) k_pcg_update(long n, const double *__restrict__ dinv, const double *__restrict__ p,
+                                                    double *__restrict__ x, int maxit, PcgWork w) {
+  if (w.sc[PCG_DONE] != PCG_RUNNING) return;
+  const double a = w.sc[PCG_ALPHA];
+  double v[2] = {0.0, 0.0}, t[2];
+  for (long i = (long)blockIdx.x * TPB + threadIdx.x; i < n; i += (long)gridDim.x * TPB) {
+    x[i] += a * p[i];
+    const double r = w.r[i] - a * w.q[i];
+    w.r[i] = r;
+    v[0] += r * r;
+    v[1] += r * (dinv[i] * r);
+  }
+  if (grid_sums<2>(v, w.partial, w.counter, t) && threadIdx.x == 0) {
+    const double rn = sqrt(t[0]), it = w.sc[PCG_ITERS] + 1.0;
+    w.sc[PCG_BETA] = t[1] / w.sc[PCG_RZ];
+    w.sc[PCG_RZ] = t[1];
+    w.sc[PCG_RNORM] = rn;
+    w.sc[PCG_ITERS] = it;
+    w.sc[PCG_DONE] = !isfinite(rn) ? PCG_NAN : rn <= w.sc[PCG_TARGET] ? PCG_CONVERGED : it >= maxit ? PCG_MAXIT : PCG_RUNNING;
+  }
 }
 
 // --------------------------------------------------------------------------
@@ -2221,11 +2317,6 @@ void vec_sub_mean(int n, T *x, const double *sum, cudaStream_t s) {
 }
 template void vec_sub_mean<double>(int, double *, const double *, cudaStream_t);
 template void vec_sub_mean<float>(int, float *, const double *, cudaStream_t);
-void vec_mul(long n, const double *a, const double *b, double *out, cudaStream_t s) {
-  k_mul<<<nblocks(n, TPB), TPB, 0, s>>>(n, a, b, out);
-  CHNSS_LAUNCH_CK();
-}
-
 void sum_partials(int nb, int k, const double *partial, double *out, cudaStream_t s) {
   k_sum_final<<<std::min(k, 64), TPB, 0, s>>>(nb, k, partial, out);
   CHNSS_LAUNCH_CK();
@@ -2458,17 +2549,23 @@ void set_scalar(double *dst, const double *src, double scale, bool sq, cudaStrea
   k_set_scalar<<<1, 1, 0, s>>>(dst, src, scale, sq ? 1 : 0);
   CHNSS_LAUNCH_CK();
 }
-void pcg_alpha(const double *rz, const double *pq, double *alpha, cudaStream_t s) {
-  k_pcg_alpha<<<1, 1, 0, s>>>(rz, pq, alpha);
+// blocks of the PCG kernels: one row a thread while the device holds them,
+// and two partials a block within the smallest buffer (kReduceMaxBlocks)
+static int pcg_blocks(long n) {
+  return (int)std::min<long>((n + TPB - 1) / TPB, std::min(8 * device_sm_count(), kReduceMaxBlocks / 2));
+}
+void pcg_start(long n, const double *dinv, const double *b, double *x, double *p, double rtol, const PcgWork &w,
+               cudaStream_t s) {
+  CHNSS_CK(cudaMemsetAsync(w.counter, 0, sizeof(int), s));
+  k_pcg_start<<<pcg_blocks(n), TPB, 0, s>>>(n, dinv, b, x, p, rtol, w);
   CHNSS_LAUNCH_CK();
 }
-void pcg_update_xr(long n, const double *alpha, const double *p, const double *q, double *x, double *r,
-                   cudaStream_t s) {
-  k_pcg_xr<<<nblocks(n, TPB), TPB, 0, s>>>(n, alpha, p, q, x, r);
+void pcg_iteration(const Pattern &P, const double *val, const double *dinv, double *x, const double *p_old,
+                   double *p_new, int maxit, const PcgWork &w, cudaStream_t s) {
+  const int nb = pcg_blocks(P.nrows);
+  k_pcg_apply<<<nb, TPB, 0, s>>>(P.nrows, P.rowptr, P.col, val, dinv, p_old, p_new, w);
   CHNSS_LAUNCH_CK();
-}
-void pcg_update_p(long n, const double *rzn, const double *rzo, const double *z, double *p, cudaStream_t s) {
-  k_pcg_p<<<nblocks(n, TPB), TPB, 0, s>>>(n, rzn, rzo, z, p);
+  k_pcg_update<<<nb, TPB, 0, s>>>(P.nrows, dinv, p_new, x, maxit, w);
   CHNSS_LAUNCH_CK();
 }
 
