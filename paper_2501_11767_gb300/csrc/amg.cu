@@ -503,6 +503,8 @@ struct AmgHandle {
     mg64.reset();
     mg32.reset();
     ar.release();
+    for (Graph *g : {&g_numeric, &g_cycle})
+      if (g->exec) cudaGraphExecDestroy(g->exec);
     if (pinned) cudaFreeHost(pinned);
     if (pinned_i) cudaFreeHost(pinned_i);
     if (s && own_stream) cudaStreamDestroy(s);
@@ -730,13 +732,55 @@ struct AmgHandle {
   }
 
   // the handle's own numeric setup: the levels, the FP64 operator of the
-  // solve and the V-cycle data, then a synchronisation
-  void numeric() {
+  // solve and the V-cycle data
+  void numeric_body() {
     levels_numeric(s);
     sell_gather<double>(lv[0]->A.sell, 1, lv[0]->val, a0sell, s);
     if (mg64) mg64->setup(s);
     else mg32->setup(s);
+  }
+  // ... followed by a synchronisation
+  void numeric() {
+    replay(g_numeric);
     CHNSS_CK(cudaStreamSynchronize(s));
+  }
+
+  // Both repeated parts, the numeric setup (about 150 launches at 512^2) and
+  // the V-cycle (about 40), as graphs: their kernels take a few microseconds
+  // each, less than the host takes to launch them one by one.
+  struct Graph {
+    cudaGraphExec_t exec = nullptr;
+    long long kernels = 0;
+  };
+  Graph g_numeric, g_cycle;
+  template <typename F>
+  void record(Graph &g, F &&body) {
+    const long long before = g_launch_count.load();
+    cudaGraph_t graph = nullptr;
+    CHNSS_CK(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+    try {
+      body();
+    } catch (...) {
+      cudaStreamEndCapture(s, &graph);
+      if (graph) cudaGraphDestroy(graph);
+      throw;
+    }
+    CHNSS_CK(cudaStreamEndCapture(s, &graph));
+    g.kernels = g_launch_count.load() - before;
+    const cudaError_t e = cudaGraphInstantiate(&g.exec, graph, 0);
+    cudaGraphDestroy(graph);
+    CHNSS_CK(e);
+  }
+  void replay(const Graph &g) {
+    CHNSS_CK(cudaGraphLaunch(g.exec, s));
+    g_launch_count.fetch_add(g.kernels, std::memory_order_relaxed);
+  }
+  void record_graphs() {
+    record(g_numeric, [&] { numeric_body(); });
+    record(g_cycle, [&] {
+      if (mg64) mg64->apply(s);
+      else mg32->apply(s);
+    });
   }
 
   template <typename T>
@@ -761,13 +805,13 @@ struct AmgHandle {
     if (mg64) {
       k_to<double><<<nblk(n0), TPB, 0, s>>>(n0, b, mg64->input());
       CHNSS_LAUNCH_CK();
-      mg64->apply(s);
+      replay(g_cycle);
       k_from<double><<<nblk(n0), TPB, 0, s>>>(n0, mg64->output(), x);
       CHNSS_LAUNCH_CK();
     } else {
       k_to<float><<<nblk(n0), TPB, 0, s>>>(n0, b, mg32->input());
       CHNSS_LAUNCH_CK();
-      mg32->apply(s);
+      replay(g_cycle);
       k_from<float><<<nblk(n0), TPB, 0, s>>>(n0, mg32->output(), x);
       CHNSS_LAUNCH_CK();
     }
@@ -920,6 +964,7 @@ chnss_status chnss_amg_create(int n, int nnz, const int *rowptr, const int *col,
   if (precision == 0) h.make_mg(h.mg64);
   else h.make_mg(h.mg32);
   h.ws.init(h.ar, kAmgRestart, n, h.pinned);
+  h.record_graphs();
   h.numeric();
   *out = H.release();
   return CHNSS_OK;
