@@ -274,9 +274,12 @@ void ch_precond(chnss_ctx *c, PrecSet<T> &P, int sp, double **slot, cudaStream_t
   const int N1 = c->N1;
   const double *const *in = const_cast<const double *const *>(slot);
   double *const *out = slot + 1;
-  vec_convert_from_slot<double, T>(N1, in, 0, P.L.input(), s);
-  P.L.apply(s);
-  P.L.write_output(out, 0, s);
+  // MG(L) beside the two cycles of the Schur part (a side branch: a third of
+  // a coarse, latency-bound preconditioner)
+  cudaStream_t q = fork_side(c, s, 0);
+  vec_convert_from_slot<double, T>(N1, in, 0, P.L.input(), q);
+  P.L.apply(q);
+  P.L.write_output(out, 0, q);
   // S~^-1 = X2^-1 M X1^-1 (matching factors of eqn::schurCH)
   MGHier<T> &X1 = P.X1[sp];
   MGHier<T> &X2 = c->p.mobility_kind == 0 ? P.X1[sp] : P.X2[sp];
@@ -286,6 +289,7 @@ void ch_precond(chnss_ctx *c, PrecSet<T> &P, int sp, double **slot, cudaStream_t
   spmv_sell<T>(c->lv(0).p1, P.Mv, 1, X1.output(), X2.input(), SPMV_PLAIN, none, s);
   X2.apply(s);
   X2.write_output(out, N1, s);
+  join_side(c, s, 0);
 }
 
 // The three species' preconditioners in one pass (slots kBatchSlot..+5):
@@ -400,6 +404,7 @@ void run_prec(chnss_ctx *c, int g, const double *r, double *z, cudaStream_t s) {
 struct CHBatchPrec : BatchPrecond {
   chnss_ctx *c;
   explicit CHBatchPrec(chnss_ctx *c_) : c(c_) {}
+  int single = -1;                  // the only species still iterating (-1: more than one)
   void apply(int K, const double *const *r, double *const *z, cudaStream_t s) override;
   void after_sync() override;
 };
@@ -414,6 +419,19 @@ void harvest_probes(chnss_ctx *c, int g) {
 }
 
 void CHBatchPrec::apply(int K, const double *const *r, double *const *z, cudaStream_t s) {
+  // the last species left runs its own preconditioner (the same bits): the
+  // batched one would still sweep the finished members' vectors
+  int active = 0;
+  for (int k = 0; k < K; ++k)
+    if (r[k]) {
+      ++active;
+      single = k;
+    }
+  if (active == 1) {
+    run_prec(c, single, r[single], z[single], s);
+    return;
+  }
+  single = -1;
   const void *ptrs[6];
   for (int k = 0; k < 3; ++k) {
     ptrs[2 * k] = k < K && r[k] ? r[k] : c->dummy_in;
@@ -430,7 +448,7 @@ void CHBatchPrec::apply(int K, const double *const *r, double *const *z, cudaStr
   g_launch_count.fetch_add(pg.nodes, std::memory_order_relaxed);
   if (prof) c->probe_pending[5] = true;
 }
-void CHBatchPrec::after_sync() { harvest_probes(c, 5); }
+void CHBatchPrec::after_sync() { harvest_probes(c, single >= 0 ? single : 5); }
 
 struct CHOp : LinearOperator {
   chnss_ctx *c;
