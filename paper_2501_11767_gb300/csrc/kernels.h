@@ -284,7 +284,8 @@ void pcg_iteration(const Pattern &P, const double *val, const double *dinv, doub
 // dense coarse-grid inverse (one CTA, Gauss-Jordan with partial pivoting)
 void coarse_dense_csr(const Pattern &P, const double *val, double add_all, double *dense, cudaStream_t s);
 void coarse_dense_bsr2(const Pattern &P, const double *val, double *dense, cudaStream_t s);
-void dense_invert(int n, double *a, double *inv, int *status, cudaStream_t s);
+// unit (may be null, n even): nonzero where rows and columns 2 i, 2 i + 1 are the identity's
+void dense_invert(int n, double *a, double *inv, int *status, cudaStream_t s, const int *unit = nullptr);
 template <typename T>
 void dense_apply(int n, const double *inv, const T *b, T *x, cudaStream_t s);
 

@@ -298,7 +298,7 @@ void MGHier<T>::setup(cudaStream_t s) {
     coarse_dense_bsr2(*pat[L], val64[L], dense, s);
   else
     coarse_dense_csr(*pat[L], val64[L], singular ? 1.0 : 0.0, dense, s);
-  dense_invert(nc, dense, cinv, status, s);
+  dense_invert(nc, dense, cinv, status, s, kind == 1 && !p2lev.empty() ? p2lev[L]->bnd2 : nullptr);
 }
 
 template <typename T>

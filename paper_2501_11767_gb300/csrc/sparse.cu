@@ -973,32 +973,60 @@ __global__ void k_combine(long n, const double *__restrict__ Z, long ldz, int k0
 }
 
 // pyth = 1: *nrm2 holds ||w||^2 after the first correction and the norm
-// after the second one is ||w||^2 - ||h2||^2 (the basis is orthonormal)
-__global__ void k_arnoldi_finish(int j, int ldh, double *H, const double *h1, const double *h2, const double *nrm2,
-                                 double *cs, double *sn, double *g, double *status, int pyth) {
-  double *col = H + (long)j * ldh;
-  for (int i = 0; i <= j; ++i) col[i] = h1[i] + h2[i];
-  double q = *nrm2;
-  if (pyth) {
-    for (int i = 0; i <= j; ++i) q -= h2[i] * h2[i];
-    q = fmax(q, 0.0);
+// after the second one is ||w||^2 - ||h2||^2 (the basis is orthonormal).
+// The recurrences are one thread's; one block stages their operands, so that
+// its loads are from shared memory (9.7 us with a dependent L2 load in every
+// step, at j = 12 on average).  At most kArnoldiMax columns.
+constexpr int kArnoldiMax = 64;
+__global__ void __launch_bounds__(kArnoldiMax) k_arnoldi_finish(int j, int ldh, double *H, const double *h1,
+                                                                const double *h2, const double *nrm2, double *cs,
+                                                                double *sn, double *g, double *status, int pyth) {
+  __shared__ double col[kArnoldiMax + 1], s2[kArnoldiMax], sc[kArnoldiMax], ss[kArnoldiMax];
+  __shared__ double gj, nr;
+  const int t = threadIdx.x;
+  double *out = H + (long)j * ldh;
+  if (t <= j) {
+    const double a = h1[t], b = h2[t];
+    col[t] = a + b;
+    s2[t] = b;
   }
-  const double hn = sqrt(q);
-  col[j + 1] = hn;
-  for (int i = 0; i < j; ++i) {
-    const double a = col[i], c = col[i + 1];
-    col[i] = cs[i] * a + sn[i] * c;
-    col[i + 1] = -sn[i] * a + cs[i] * c;
+  if (t < j) {
+    sc[t] = cs[t];
+    ss[t] = sn[t];
   }
-  const double den = hypot(col[j], col[j + 1]);
-  cs[j] = col[j] / den;
-  sn[j] = col[j + 1] / den;
-  col[j] = den;
-  col[j + 1] = 0.0;
-  g[j + 1] = -sn[j] * g[j];
-  g[j] = cs[j] * g[j];
-  status[0] = fabs(g[j + 1]);
-  status[1] = hn;
+  if (t == 0) {
+    gj = g[j];
+    nr = *nrm2;
+  }
+  __syncthreads();
+  if (t == 0) {
+    double q = nr;
+    if (pyth) {
+      for (int i = 0; i <= j; ++i) q -= s2[i] * s2[i];
+      q = fmax(q, 0.0);
+    }
+    const double hn = sqrt(q);
+    col[j + 1] = hn;
+    for (int i = 0; i < j; ++i) {
+      const double a = col[i], c = col[i + 1];
+      col[i] = sc[i] * a + ss[i] * c;
+      col[i + 1] = -ss[i] * a + sc[i] * c;
+    }
+    const double den = hypot(col[j], col[j + 1]);
+    const double cj = col[j] / den, sj = col[j + 1] / den;
+    cs[j] = cj;
+    sn[j] = sj;
+    col[j] = den;
+    col[j + 1] = 0.0;
+    const double gn = -sj * gj;
+    g[j + 1] = gn;
+    g[j] = cj * gj;
+    status[0] = fabs(gn);
+    status[1] = hn;
+  }
+  __syncthreads();
+  if (t <= j) out[t] = col[t];
+  if (t == 0) out[j + 1] = 0.0;
 }
 
 __global__ void k_hessenberg_solve(int k0, const int *kd, int ldh, const double *H, const double *g, double *y) {
@@ -1165,6 +1193,9 @@ __global__ void k_dense_bsr2(int nrows, const int *rowptr, const int *col, const
 // step).  Every block finds the pivot from its own copy of the column.
 // Columns that are still (or already) unit vectors are left out: their
 // pivot-row entry is zero.  Entry by entry the operations of k_dense_invert.
+// unit (may be null): nonzero where the pair of rows 2 i, 2 i + 1 and its
+// columns are the identity's (nodes with prescribed velocity): such a step
+// changes nothing and is not taken (242 rows: 162 steps).
 // The cluster barrier and the pivot's division now bound the step.
 constexpr int kInvCtas = 16;
 constexpr int kInvThreads = 512;
@@ -1174,6 +1205,7 @@ struct InvSmem {
   double prow[2 * kCoarseDenseMax / kInvCtas];        // pivot row of the block's columns
   int used[kCoarseDenseMax];                          // original rows taken as pivots
   int orig[kCoarseDenseMax];                          // original row at each position
+  int unit[kCoarseDenseMax];                          // rows and columns of the identity
   int act[2 * kCoarseDenseMax / kInvCtas];            // the block's columns with work in this step
   int nact, piv;
 };
@@ -1182,7 +1214,8 @@ inline size_t inv_smem_bytes(int n) {
   return sizeof(InvSmem) + (size_t)2 * lc * n * sizeof(double);
 }
 __global__ void __launch_bounds__(kInvThreads) k_dense_invert_cluster(int n, const double *__restrict__ a,
-                                                                      double *__restrict__ inv, int *status) {
+                                                                      double *__restrict__ inv, int *status,
+                                                                      const int *__restrict__ unit) {
   extern __shared__ __align__(16) unsigned char raw[];
   InvSmem &S = *reinterpret_cast<InvSmem *>(raw);
   double *W = reinterpret_cast<double *>(raw + sizeof(InvSmem));   // [2 lc][n]: a columns, then inv columns
@@ -1195,14 +1228,23 @@ __global__ void __launch_bounds__(kInvThreads) k_dense_invert_cluster(int n, con
     W[(lc + j) * n + r] = r == q ? 1.0 : 0.0;
   }
   for (int r = tid; r < n; r += kInvThreads) {
-    S.col[0][r] = a[(long)r * n];
     S.used[r] = 0;
     S.orig[r] = r;
+    S.unit[r] = unit ? unit[r >> 1] : 0;
   }
+  __syncthreads();
+  auto next_column = [&](int c) {   // the next one that is not a unit vector
+    while (c < n && S.unit[c]) ++c;
+    return c;
+  };
+  const int c_first = next_column(0);
+  for (int r = tid; r < n && c_first < n; r += kInvThreads) S.col[0][r] = a[(long)r * n + c_first];
   bool zero = false;
   cl.sync();
-  for (int c = 0; c < n; ++c) {
-    double *cb = S.col[c & 1];
+  int buf = 0;
+  for (int c = c_first; c < n;) {
+    const int cn = next_column(c + 1);
+    double *cb = S.col[buf];
     if (tid < 32) {   // pivot: largest magnitude, first row among equals; then this step's columns
       double best = -1.0;
       int bi = c;
@@ -1224,10 +1266,10 @@ __global__ void __launch_bounds__(kInvThreads) k_dense_invert_cluster(int n, con
         S.used[t] = 1;
       }
       __syncwarp();
-      int na = 0;   // the next pivot column first, so that it can leave early
+      int na = 0;
       for (int j0 = 0; j0 < 2 * lc; j0 += 32) {
         const int j = j0 + tid, q = (j < lc ? j : j - lc) * kInvCtas + me;
-        const bool on = j < 2 * lc && q < n && (j < lc ? q > c : S.used[q] != 0);
+        const bool on = j < 2 * lc && q < n && (j < lc ? q > c && !S.unit[q] : S.used[q] != 0);
         const unsigned m = __ballot_sync(0xffffffffu, on);
         if (on) S.act[na + __popc(m & ((1u << tid) - 1u))] = j;
         na += __popc(m);
@@ -1259,7 +1301,7 @@ __global__ void __launch_bounds__(kInvThreads) k_dense_invert_cluster(int n, con
     __syncthreads();
     const int rows = (n + 31) / 32 * 32, groups = kInvThreads / rows;
     const int g = tid / rows, r = tid % rows;
-    const bool mine = c + 1 < n && (c + 1) % kInvCtas == me;   // act[0] is column c + 1 then
+    const bool mine = cn < n && cn % kInvCtas == me;
     if (g < groups && r < n && r != c) {
       const double f = cb[r];
       for (int k = g; k < na; k += groups) {
@@ -1269,11 +1311,13 @@ __global__ void __launch_bounds__(kInvThreads) k_dense_invert_cluster(int n, con
     }
     if (mine) {
       __syncthreads();
-      const double *w = W + ((c + 1) / kInvCtas) * n;
+      const double *w = W + (cn / kInvCtas) * n;
       for (int t = tid; t < n * kInvCtas; t += kInvThreads)
-        cl.map_shared_rank(&S.col[(c + 1) & 1][0], t / n)[t % n] = w[t % n];
+        cl.map_shared_rank(&S.col[buf ^ 1][0], t / n)[t % n] = w[t % n];
     }
     cl.sync();
+    c = cn;
+    buf ^= 1;
   }
   for (int t = tid; t < lc * n; t += kInvThreads) {
     const int r = t / lc, j = t % lc, q = j * kInvCtas + me;
@@ -2383,12 +2427,12 @@ void combine_columns_dev(long n, const double *Z, long ldz, const int *k, const 
 }
 void arnoldi_finish(int j, int ldh, double *H, const double *h1, const double *h2, const double *nrm2, double *cs,
                     double *sn, double *g, double *status, cudaStream_t s) {
-  k_arnoldi_finish<<<1, 1, 0, s>>>(j, ldh, H, h1, h2, nrm2, cs, sn, g, status, 0);
+  k_arnoldi_finish<<<1, kArnoldiMax, 0, s>>>(j, ldh, H, h1, h2, nrm2, cs, sn, g, status, 0);
   CHNSS_LAUNCH_CK();
 }
 void arnoldi_finish_pyth(int j, int ldh, double *H, const double *h1, const double *h2w, double *cs, double *sn,
                          double *g, double *status, cudaStream_t s) {
-  k_arnoldi_finish<<<1, 1, 0, s>>>(j, ldh, H, h1, h2w, h2w + j + 1, cs, sn, g, status, 1);
+  k_arnoldi_finish<<<1, kArnoldiMax, 0, s>>>(j, ldh, H, h1, h2w, h2w + j + 1, cs, sn, g, status, 1);
   CHNSS_LAUNCH_CK();
 }
 
@@ -2577,12 +2621,12 @@ void coarse_dense_bsr2(const Pattern &P, const double *val, double *dense, cudaS
   k_dense_bsr2<<<P.nrows, 128, 0, s>>>(P.nrows, P.rowptr, P.col, val, dense);
   CHNSS_LAUNCH_CK();
 }
-void dense_invert(int n, double *a, double *inv, int *status, cudaStream_t s) {
+void dense_invert(int n, double *a, double *inv, int *status, cudaStream_t s, const int *unit) {
   if (n <= kCoarseDenseMax) {
     constexpr size_t most = sizeof(InvSmem) + 2 * (kCoarseDenseMax / kInvCtas) * kCoarseDenseMax * sizeof(double);
     allow_cluster<k_dense_invert_cluster>(most);
     launch_cluster(k_dense_invert_cluster, kInvCtas, 1, kInvThreads, inv_smem_bytes(n), s, n, (const double *)a, inv,
-                   status);
+                   status, unit);
     CHNSS_LAUNCH_CK();
     return;
   }
