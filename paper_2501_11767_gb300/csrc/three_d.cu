@@ -956,6 +956,9 @@ struct chnss3_ctx {
   // captured preconditioners (0..2 CH species, 3 AC, 4 Oseen) replayed from
   // fixed staging vectors; each captured on a private stream of its own
   cudaStream_t cap[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+  // their side branches (independent parts of one preconditioner)
+  cudaStream_t side[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+  cudaEvent_t ev_fork[5] = {}, ev_join[5] = {};
   // bodies of the inner multigrid loops (inner_rtol > 0), one stream per solve group
   cudaStream_t bodyq[3] = {nullptr, nullptr, nullptr};
   cudaGraphExec_t gexec[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
@@ -974,6 +977,12 @@ struct chnss3_ctx {
       if (g) cudaGraphExecDestroy(g);
     for (cudaStream_t q : cap)
       if (q) cudaStreamDestroy(q);
+    for (cudaStream_t q : side)
+      if (q) cudaStreamDestroy(q);
+    for (int g = 0; g < 5; ++g) {
+      if (ev_fork[g]) cudaEventDestroy(ev_fork[g]);
+      if (ev_join[g]) cudaEventDestroy(ev_join[g]);
+    }
     for (cudaStream_t q : bodyq)
       if (q) cudaStreamDestroy(q);
     for (cudaStream_t q : sx)
@@ -1284,6 +1293,11 @@ void create3(chnss3_ctx *c, int n) {
   CHNSS_CK(cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high));
   for (int w = 0; w < 3; ++w)
     CHNSS_CK(cudaStreamCreateWithPriority(&c->sx[w], cudaStreamNonBlocking, w == 2 ? prio_high : prio_low));
+  for (int g = 0; g < 5; ++g) {
+    CHNSS_CK(cudaStreamCreateWithFlags(&c->side[g], cudaStreamNonBlocking));
+    CHNSS_CK(cudaEventCreateWithFlags(&c->ev_fork[g], cudaEventDisableTiming));
+    CHNSS_CK(cudaEventCreateWithFlags(&c->ev_join[g], cudaEventDisableTiming));
+  }
   CHNSS_CK(cudaEventCreateWithFlags(&c->ev_asm, cudaEventDisableTiming));
   for (cudaEvent_t &e : c->ev_done) CHNSS_CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   c->mt0 = ar.alloc<double>(N1);
@@ -1471,10 +1485,23 @@ void mg_apply(MGHier<T> &h, long n, const double *r, double *z, cudaStream_t s) 
   mg_output(h, n, z, s);
 }
 
+// Side branch of preconditioner g's graph, forked off s and joined back
+// (s is capturing: its levels are latency bound, so independent V-cycles run
+// beside each other).
+cudaStream_t fork3(chnss3_ctx *c, int g, cudaStream_t s) {
+  CHNSS_CK(cudaEventRecord(c->ev_fork[g], s));
+  CHNSS_CK(cudaStreamWaitEvent(c->side[g], c->ev_fork[g], 0));
+  return c->side[g];
+}
+void join3(chnss3_ctx *c, int g, cudaStream_t s) {
+  CHNSS_CK(cudaEventRecord(c->ev_join[g], c->side[g]));
+  CHNSS_CK(cudaStreamWaitEvent(s, c->ev_join[g], 0));
+}
+
 template <typename T>
 void prec_ch3(chnss3_ctx *c, Prec3<T> &P, int sp, const double *r, double *z, cudaStream_t s) {
   const long N1 = c->lv[0].N1;
-  mg_apply(P.L, N1, r, z, s);
+  mg_apply(P.L, N1, r, z, fork3(c, sp, s));
   // S~^-1 = X2^-1 M X1^-1 (matching factors of eqn::schurCH; X2 = X1 with
   // constant mobility)
   MGHier<T> &X1 = P.X[sp], &X2 = c->p.mobility_kind != 0 ? P.X2[sp] : P.X[sp];
@@ -1484,19 +1511,20 @@ void prec_ch3(chnss3_ctx *c, Prec3<T> &P, int sp, const double *r, double *z, cu
   spmv_sell<T>(c->lv[0].p1, P.Ms, 1, X1.output(), X2.input(), SPMV_PLAIN, none, s);
   X2.apply(s);
   mg_output(X2, N1, z + N1, s);
+  join3(c, sp, s);
 }
 
 template <typename T>
 void prec_ns3(chnss3_ctx *c, Prec3<T> &P, const double *r, double *z, cudaStream_t s) {
   const Level3 &F = c->lv[0];
   const long nv = 3 * F.N2, N1 = F.N1;
-  mg_apply(P.A, nv, r, z, s);
-  // pressure convection-diffusion: M_p^-1 A_p K_p^-1
-  vec_convert<double, T>(N1, r + nv, P.Kp.input(), s);
-  P.Kp.apply(s);
+  // pressure convection-diffusion M_p^-1 A_p K_p^-1 beside the velocity block
+  cudaStream_t q = fork3(c, 4, s);
+  vec_convert<double, T>(N1, r + nv, P.Kp.input(), q);
+  P.Kp.apply(q);
   SpmvArgs none;
-  spmv_sell<T>(F.p1, P.Aps, 1, P.Kp.output(), P.mb, SPMV_PLAIN, none, s);
-  vec_scale_dinv<T>((int)N1, c->massc, P.mdinv, P.mb, P.mx, s);
+  spmv_sell<T>(F.p1, P.Aps, 1, P.Kp.output(), P.mb, SPMV_PLAIN, none, q);
+  vec_scale_dinv<T>((int)N1, c->massc, P.mdinv, P.mb, P.mx, q);
   SpmvArgs a;
   a.b = P.mb;
   a.dinv = P.mdinv;
@@ -1504,10 +1532,12 @@ void prec_ns3(chnss3_ctx *c, Prec3<T> &P, const double *r, double *z, cudaStream
   for (int k = 1; k <= 4; ++k) {
     a.coef = c->massc + 1 + 3 * (k - 1);
     a.w = k == 1 ? nullptr : other;
-    spmv_sell<T>(F.p1, P.Ms, 1, cur, other, SPMV_CHEB, a, s);
+    spmv_sell<T>(F.p1, P.Ms, 1, cur, other, SPMV_CHEB, a, q);
     std::swap(cur, other);
   }
-  vec_convert<T, double>(N1, cur, z + nv, s);
+  vec_convert<T, double>(N1, cur, z + nv, q);
+  mg_apply(P.A, nv, r, z, s);
+  join3(c, 4, s);
 }
 
 void prec_body3(chnss3_ctx *c, int g, const double *r, double *z, cudaStream_t s) {
