@@ -309,7 +309,7 @@ __global__ void k_p2_check(int n, int open, const int *__restrict__ rowptr, cons
 constexpr int kCount = 2 * (kP2Slots + kP2TopSlots);
 
 bool p2_applies(const Level &L, const P2Table &t, size_t value_size) {
-  return t.ok && (value_size < 8 || sell_warps_bsr2(L.p2.sell) == 1);
+  return t.ok && value_size < 8;
 }
 
 P2Table p2_table(Arena &keep, const Level &L, int open_top, const double *A, cudaStream_t s) {

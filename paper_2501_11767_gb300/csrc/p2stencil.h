@@ -34,11 +34,12 @@ inline long p2_ld(int n) { return ((long)(n + 1) * (n + 1) + 31) / 32 * 32; }
 inline long p2_values_count(int n) { return 2 * kP2Slots * p2_ld(n); }   // scalars
 
 // Whether a level with table t takes the stencil for values of value_size
-// bytes: always in FP32 and BF16 (384^2: fine level 31.0 -> 18.0 us a sweep,
-// 192^2 level 12.1 -> 10.9, coarser ones 6.1 -> 4.4-5.1), in FP64 from the
-// size on at which a row is one thread's (n = 241).  Below it an FP64 sweep
-// is bound by its arithmetic and its latencies, and the SELL kernel with
-// several warps a slice is the faster one (128^2: 16.5 against 18.7 us).
+// bytes: in FP32 and BF16 (384^2: fine level 31.0 -> 18.0 us a sweep, 192^2
+// level 12.1 -> 10.9, coarser ones 6.1 -> 4.4-5.1).  FP64 sweeps stay on the
+// 2x2-block SELL: they are bound by the FP64 pipe, not by the bytes saved, and
+// the stencil's fewer, longer threads keep it less busy (FP64 steps with the
+// stencil from 241^2 on against SELL: 512^2 137 and 131 ms, 768^2 287 and 267,
+// 1024^2 497 and 460; a sweep of 128^2 18.7 and 16.5 us).
 bool p2_applies(const Level &L, const P2Table &t, size_t value_size);
 // Table of the level's constant blocks A (CSR order, 4 values each) and
 // whether all its rows match it (synchronises s); device copies from keep.
@@ -59,8 +60,9 @@ template <typename T, typename VT>
 void p2_spmv(const Level &L, int open_top, const P2Table &tab, const VT *val, const T *u, T *out, SpmvMode mode,
              const SpmvArgs &a, P2Start start, const double *scale, cudaStream_t s);
 
-// b = R r onto the mesh of nc cells a side; x += P xc from it (velocity
-// transfers of build_vel_transfer, the same sums; vectors aligned to a node)
+// b = R r onto the mesh of nc cells a side; x += P xc from it: quadratic
+// interpolation between the nodes without prescribed velocity of both meshes
+// and its transpose (vectors aligned to a node)
 template <typename T>
 void p2_restrict(int nc, int open_top, const T *r, T *b, cudaStream_t s);
 template <typename T>
