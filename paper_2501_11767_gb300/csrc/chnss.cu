@@ -572,14 +572,13 @@ void init_precset(chnss_ctx *c, PrecSet<T> &P) {
   const int nl = c->nlev;
   std::vector<const Pattern *> p1s, p2s;
   std::vector<const int *> d1s, d2s;
-  std::vector<const Transfer *> t1s, tvs;
+  std::vector<const Transfer *> t1s;
   for (int l = 0; l < nl; ++l) {
     p1s.push_back(&c->lv(l).p1);
     p2s.push_back(&c->lv(l).p2);
     d1s.push_back(c->lv(l).diag1);
     d2s.push_back(c->lv(l).diag2);
     t1s.push_back(&c->lv(l).t1);
-    tvs.push_back(&c->lv(l).tv);
   }
   auto vals = [&](const std::vector<double *> &v) { return std::vector<const double *>(v.begin(), v.end()); };
   // precision 2: BF16 values for the velocity hierarchy, where they cut the
@@ -608,7 +607,7 @@ void init_precset(chnss_ctx *c, PrecSet<T> &P) {
   P.A.open_top = c->mesh->m.top_bc;
   P.A.degree = 4;        // velocity smoothing: degree 4 on [hi / 16, hi]
   P.A.ratio = 16.0;
-  P.A.init(ar, 1, false, p2s, d2s, vals(c->A), tvs, c->partial);
+  P.A.init(ar, 1, false, p2s, d2s, vals(c->A), {}, c->partial);   // transfers: p2lev
   // the fine operator applied inside FGMRES: in stencil order it is the FP64
   // hierarchy's own level 0, or a copy written together with the FP32 values
   if (c->p2fine() && std::is_same<T, double>::value)
@@ -2405,8 +2404,6 @@ void set_block(chnss_ctx *c, bool velocity, int block) {
   for (Level &L : m.lv) {
     if (velocity) {
       L.p2.sell.block = block;
-      L.tv.P.sell.block = block;
-      L.tv.R.sell.block = block;
     } else {
       L.p1.sell.block = block;
       L.t1.P.sell.block = block;

@@ -157,7 +157,6 @@ struct Level {
   int *diag1 = nullptr;  // [N1] position of the diagonal in p1
   int *diag2 = nullptr;  // [N2] position of the diagonal block in p2
   Transfer t1;           // P1 transfer from level+1 (empty on the coarsest)
-  Transfer tv;           // velocity (per node, masked) transfer from level+1
 };
 
 struct Mesh {

@@ -132,7 +132,7 @@ struct TailDesc {
 };
 // width: 8 or 16, the widest row of any tail operator or transfer (rounded up)
 template <typename T>
-void mg_tail(const TailDesc<T> *d_desc, int nr, int width, cudaStream_t s);
+void mg_tail(const TailDesc<T> *d_desc, int width, cudaStream_t s);
 // BF16-stored values, FP32 vectors and accumulation (preconditioner variant)
 void spmv_sell(const Pattern &P, const __nv_bfloat16 *sval, int ncomp, const float *u, float *out, SpmvMode mode,
                const SpmvArgs &a, cudaStream_t s);

@@ -247,47 +247,6 @@ void build_p1_transfer(Arena &ar, int nc, Transfer &t) {
   finish_transfer(ar, t, pv);
 }
 
-// Quadratic interpolation of coarse P2 functions at the fine P2 nodes, on
-// the nodes without prescribed velocity of both levels (open top: the top
-// edge except its corners is free).
-void build_vel_transfer(Arena &ar, int nc, int top_bc, Transfer &t) {
-  const int mf = 4 * nc + 1, mc = 2 * nc + 1;
-  Pattern &P = t.P;
-  P.nrows = mf * mf;
-  P.ncols = mc * mc;
-  P.h_rowptr.assign(P.nrows + 1, 0);
-  std::vector<double> pv;
-  auto cbnd = [&](int id) {
-    int I = id % mc, J = id / mc;
-    return I == 0 || J == 0 || I == mc - 1 || (top_bc == 0 && J == mc - 1);
-  };
-  for (int J = 0; J < mf; ++J)
-    for (int I = 0; I < mf; ++I) {
-      const int r = J * mf + I;
-      const bool fb = I == 0 || J == 0 || I == mf - 1 || (top_bc == 0 && J == mf - 1);
-      if (!fb) {
-        const int i = std::min(I / 4, nc - 1), j = std::min(J / 4, nc - 1);
-        const double xi = I / 4.0 - i, eta = J / 4.0 - j;   // exact quarters
-        const bool lower = xi >= eta;
-        double l[3];
-        if (lower) { l[0] = 1 - xi; l[1] = xi - eta; l[2] = eta; }
-        else       { l[0] = 1 - eta; l[1] = xi; l[2] = eta - xi; }
-        int v1[3], v2[6];
-        element_nodes(nc, 2 * (j * nc + i) + (lower ? 0 : 1), v1, v2);
-        const double w[6] = {l[0] * (2 * l[0] - 1), l[1] * (2 * l[1] - 1), l[2] * (2 * l[2] - 1),
-                             4 * l[1] * l[2], 4 * l[0] * l[2], 4 * l[0] * l[1]};
-        std::vector<std::pair<int, double>> row;
-        for (int k = 0; k < 6; ++k)
-          if (w[k] != 0.0 && !cbnd(v2[k])) row.push_back({v2[k], w[k]});
-        std::sort(row.begin(), row.end());
-        for (auto &cw : row) { P.h_col.push_back(cw.first); pv.push_back(cw.second); }
-      }
-      P.h_rowptr[r + 1] = (int)P.h_col.size();
-    }
-  P.nnz = (int)P.h_col.size();
-  finish_transfer(ar, t, pv);
-}
-
 }  // namespace
 
 void build_mesh(Mesh &m, int n, double lx, double ly, int top_bc) {
@@ -360,8 +319,7 @@ void build_mesh(Mesh &m, int n, double lx, double ly, int top_bc) {
     }
   }
   for (size_t l = 0; l + 1 < sizes.size(); ++l) {
-    build_p1_transfer(ar, sizes[l + 1], m.lv[l].t1);
-    build_vel_transfer(ar, sizes[l + 1], top_bc, m.lv[l].tv);
+    build_p1_transfer(ar, sizes[l + 1], m.lv[l].t1);   // the velocity's are computed (p2stencil.h)
   }
 }
 

@@ -362,7 +362,7 @@ void MGHier<T>::vcycle(int l, cudaStream_t s) {
     return;
   }
   if (l == tail_l0) {
-    mg_tail<T>(tail, 1, tail_width, s);
+    mg_tail<T>(tail, tail_width, s);
     return;
   }
   if (l == nl - 1 && !coarse_iter) {
@@ -380,7 +380,6 @@ void MGHier<T>::vcycle(int l, cudaStream_t s) {
     cheb_block_bsr3<T, T>(*bpat[l], val[l], dinv[l], b[l], x[l], t[l], coef[l], kCoarseDegree, s);
     return;
   }
-  const int nc_ = kind == 1 ? 2 : 1;   // transfers per node (BSR2) or per dof
   SpmvArgs a;
   a.b = b[l];
   a.dinv = dinv[l];
@@ -407,17 +406,15 @@ void MGHier<T>::vcycle(int l, cudaStream_t s) {
   SpmvArgs ar;
   ar.b = b[l];
   op(l, x[l], r[l], SPMV_RES, ar, s);
-  const Transfer &T_ = *tr[l];
   SpmvArgs none;
-  const bool p2 = kind == 1 && !p2lev.empty();   // structured velocity transfers
-  if (p2) p2_restrict<T>(p2lev[l + 1]->n, open_top, r[l], b[l + 1], s);
-  else spmv_sell<T>(T_.R, transfer_vals<T>(T_, true), nc_, r[l], b[l + 1], SPMV_PLAIN, none, s);
+  if (kind == 1) p2_restrict<T>(p2lev[l + 1]->n, open_top, r[l], b[l + 1], s);
+  else spmv_sell<T>(tr[l]->R, transfer_vals<T>(*tr[l], true), 1, r[l], b[l + 1], SPMV_PLAIN, none, s);
   const int kc = kind == 0 ? Profiler::P1_MG_COARSE : Profiler::VEL_MG_COARSE;
   const int tkc = prof && l == 0 ? prof->start(kc, s) : -1;
   vcycle(l + 1, s);
   if (prof && l == 0) prof->stop(kc, tkc, s, 0.0);   // time only: every level below the finest
-  if (p2) p2_prolong_add<T>(p2lev[l + 1]->n, open_top, x[l + 1], x[l], s);
-  else spmv_sell<T>(T_.P, transfer_vals<T>(T_, false), nc_, x[l + 1], x[l], SPMV_ADD, none, s);
+  if (kind == 1) p2_prolong_add<T>(p2lev[l + 1]->n, open_top, x[l + 1], x[l], s);
+  else spmv_sell<T>(tr[l]->P, transfer_vals<T>(*tr[l], false), 1, x[l + 1], x[l], SPMV_ADD, none, s);
   // post-smoothing from x_0 = x[l]
   a.coef = coef[l] + 1;
   a.w = nullptr;
@@ -644,10 +641,7 @@ void MGBatch<T>::init(Arena &ar, MGHier<T> *hier, int nr_) {
       r[l].p[k] = ar.alloc<T>(h->n[l]);
       b[l].p[k] = ar.alloc<T>(h->n[l]);
     }
-  if (h->mgc.first >= 0)
-    mgc = mgc_plan<T>(ar, nr, h->pat, h->tr, h->val, h->dinv, h->coef, b, x, h->degree, h->coarse_iter, h->nc, h->cinv);
-  else if (h->tail_l0 > 0)
-    tail = h->make_tail(ar, x, t, r, b);
+  mgc = mgc_plan<T>(ar, nr, h->pat, h->tr, h->val, h->dinv, h->coef, b, x, h->degree, h->coarse_iter, h->nc, h->cinv);
 }
 
 template <typename T>
@@ -674,10 +668,6 @@ void MGBatch<T>::vcycle(int l, cudaStream_t s) {
   const int nl = h->nl;
   if (l == mgc.first) {
     mgc_apply(mgc, s);
-    return;
-  }
-  if (l == h->tail_l0) {
-    mg_tail<T>(tail, nr, h->tail_width, s);
     return;
   }
   if (l == nl - 1 && !h->coarse_iter) {

@@ -74,7 +74,8 @@ struct MGHier {
   std::vector<const Transfer *> tr;
   std::vector<const Pattern *> bpat;   // kind 2: node patterns (3x3-block SELL) per level
   std::vector<const int *> bmap;       // kind 2: their map9 (value -> CSR position)
-  // kind 1 (set before init): mesh levels and stencil tables; a level that
+  // kind 1 (set before init): mesh levels (they define the transfers) and
+  // stencil tables; a level that
   // p2_applies() to is swept as a P2 stencil, any other one as 2x2-block SELL
   std::vector<const Level *> p2lev;
   std::vector<P2Table> p2tab;
@@ -180,8 +181,7 @@ struct MGBatch {
   MGHier<T> *h = nullptr;
   int nr = 0;
   std::vector<MultiPtr<T>> x, t, r, b;     // per level
-  TailDesc<T> *tail = nullptr;             // device, levels h->tail_l0..
-  MgcPlan<T> mgc;                          // or levels mgc.first.. by a cluster
+  MgcPlan<T> mgc;                          // levels mgc.first.. by a cluster
   void init(Arena &ar, MGHier<T> *hier, int nr);
   T *input(int k) { return b[0].p[k]; }
   T *output(int k) { return x[0].p[k]; }

@@ -2697,28 +2697,14 @@ template void dense_apply_multi<float>(int, int, const double *, const MultiPtr<
                                        cudaStream_t);
 
 template <typename T>
-void mg_tail(const TailDesc<T> *d_desc, int nr, int width, cudaStream_t s) {
-  if (width != 8 && width != 16) throw Error{CHNSS_ERR_ARG, "coarse-level block: rows of 8 or 16 entries"};
-  const bool w16 = width == 16;
-  switch (nr) {
-    case 1:
-      if (w16) k_mg_tail<T, 1, 16><<<1, 512, 0, s>>>(d_desc);
-      else k_mg_tail<T, 1, 8><<<1, 512, 0, s>>>(d_desc);
-      break;
-    case 2:
-      if (w16) k_mg_tail<T, 2, 16><<<1, 512, 0, s>>>(d_desc);
-      else k_mg_tail<T, 2, 8><<<1, 512, 0, s>>>(d_desc);
-      break;
-    case 3:
-      if (w16) k_mg_tail<T, 3, 16><<<1, 512, 0, s>>>(d_desc);
-      else k_mg_tail<T, 3, 8><<<1, 512, 0, s>>>(d_desc);
-      break;
-    default: throw Error{CHNSS_ERR_ARG, "coarse-level block: 1 to 3 vectors"};
-  }
+void mg_tail(const TailDesc<T> *d_desc, int width, cudaStream_t s) {
+  if (width == 8) k_mg_tail<T, 1, 8><<<1, 512, 0, s>>>(d_desc);
+  else if (width == 16) k_mg_tail<T, 1, 16><<<1, 512, 0, s>>>(d_desc);
+  else throw Error{CHNSS_ERR_ARG, "coarse-level block: rows of 8 or 16 entries"};
   CHNSS_LAUNCH_CK();
 }
-template void mg_tail<double>(const TailDesc<double> *, int, int, cudaStream_t);
-template void mg_tail<float>(const TailDesc<float> *, int, int, cudaStream_t);
+template void mg_tail<double>(const TailDesc<double> *, int, cudaStream_t);
+template void mg_tail<float>(const TailDesc<float> *, int, cudaStream_t);
 
 template <typename T>
 void vec_copy_multi(long n, int nr, const MultiPtr<T> &in, const MultiPtr<T> &out, cudaStream_t s) {
