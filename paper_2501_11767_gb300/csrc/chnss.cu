@@ -148,10 +148,7 @@ struct chnss_ctx {
   double *Apb = nullptr, *Ap = nullptr, *Bv = nullptr, *Btv = nullptr, *dinvM = nullptr;
   // SELL-ordered copies of the fine FP64 operators applied inside FGMRES
   double *Ls = nullptr, *ACs = nullptr, *As = nullptr, *Ks = nullptr, *Ms = nullptr, *Bs = nullptr, *Bts = nullptr;
-  // velocity operator as a P2 stencil (As, AsT in stencil order where level 0
-  // takes it, in 2x2-block SELL order otherwise)
-  std::vector<P2Table> p2tab;
-  bool p2fine() const { return p2_applies(lv(0), p2tab[0], sizeof(double)); }
+  std::vector<P2Table> p2tab;   // velocity levels as P2 stencils (FP32, BF16 sweeps)
   double *Kks[3] = {nullptr, nullptr, nullptr};
   double *Kk[3] = {nullptr, nullptr, nullptr};
   double *loads = nullptr, *G = nullptr, *fa = nullptr, *tmp = nullptr, *sum = nullptr, *partial = nullptr;
@@ -497,14 +494,11 @@ struct ACOp : LinearOperator {
   void after_sync() override { harvest_probes(c, 3); }
 };
 
-// y = A x on the fine velocity block (values in the layout of c->As)
+// y = A x on the fine velocity block (2x2-block SELL values)
 void apply_velocity(chnss_ctx *c, const double *val, const double *x, double *y, cudaStream_t s) {
   const Level &F = c->lv(0);
   SpmvArgs none;
-  if (c->p2fine())
-    p2_spmv<double, double>(F, c->mesh->m.top_bc, c->p2tab[0], val, x, y, SPMV_PLAIN, none, P2_PLAIN, nullptr, s);
-  else
-    spmv_sell_bsr2<double>(F.p2, val, x, y, SPMV_PLAIN, none, s);
+  spmv_sell_bsr2<double>(F.p2, val, x, y, SPMV_PLAIN, none, s);
 }
 
 struct NSOp : LinearOperator {
@@ -517,7 +511,7 @@ struct NSOp : LinearOperator {
     const int tk = c->prof.start(Profiler::NS_OUTER_SPMV, s);
     apply_velocity(c, c->As, x, y, s);
     c->prof.stop(Profiler::NS_OUTER_SPMV, tk, s,
-                 (c->p2fine() ? (double)p2.nnz * 16.0 : (double)p2.nnz * 36.0 + 4.0 * (p2.nrows + 1)) + 2.0 * nv * 8.0);
+                 (double)p2.nnz * 36.0 + 4.0 * (p2.nrows + 1) + 2.0 * nv * 8.0);
     spmv_sell_bt_add(c->mesh->m.pbt, c->Bts, x + nv, y, s);
     spmv_sell_b(c->mesh->m.pb, c->Bs, x, y + nv, s);
   }
@@ -608,14 +602,7 @@ void init_precset(chnss_ctx *c, PrecSet<T> &P) {
   P.A.degree = 4;        // velocity smoothing: degree 4 on [hi / 16, hi]
   P.A.ratio = 16.0;
   P.A.init(ar, 1, false, p2s, d2s, vals(c->A), {}, c->partial);   // transfers: p2lev
-  // the fine operator applied inside FGMRES: in stencil order it is the FP64
-  // hierarchy's own level 0, or a copy written together with the FP32 values
-  if (c->p2fine() && std::is_same<T, double>::value)
-    c->As = reinterpret_cast<double *>(P.A.val[0]);
-  else if (c->p2fine())
-    c->As = P.A.copy64 = ar.alloc<double>(p2_values_count(c->lv(0).n));
-  else
-    c->As = ar.alloc<double>(4L * c->lv(0).p2.sell.nent);
+  c->As = ar.alloc<double>(4L * c->lv(0).p2.sell.nent);   // the fine operator applied inside FGMRES
   P.Kp.keep_dense = true;       // a pure Laplacian: its coarsest level is not mass-dominated
   if (c->mesh->m.top_bc == 1)   // open top: Dirichlet outflow rows, non-singular
     P.Kp.init(ar, 0, false, p1s, d1s, vals(c->Kpd), t1s, c->partial);
@@ -994,7 +981,7 @@ void assemble_ns(chnss_ctx *c, const chnss_state *st, const AsmLevels &lv, cudaS
   spmv_csr<double>(F.p2, c->M2v[0], 2, st->v, c->rhs[5], SPMV_PLAIN, none, s);
   vec_axpby(nv, 1.0, c->G, 1.0 / p.tau, c->rhs[5], s);
   vec_fill(N1, 0.0, c->rhs[5] + nv, s);
-  if (!c->p2fine()) sell_gather<double>(F.p2.sell, 4, c->A[0], c->As, s);
+  sell_gather<double>(F.p2.sell, 4, c->A[0], c->As, s);
   if (c->p32) setup_step_precset_ns(c, *c->p32, s);
   else setup_step_precset_ns(c, *c->p64, s);
 }
@@ -2048,7 +2035,7 @@ void adjoint_alloc(chnss_ctx *c) {
   const long N1 = c->N1, nmax = 2L * c->N2 + c->N1;
   c->LsT = ar.alloc<double>(F.p1.sell.nent);
   c->ACsT = ar.alloc<double>(F.p1.sell.nent);
-  c->AsT = ar.alloc<double>(c->p2fine() ? p2_values_count(F.n) : 4L * F.p2.sell.nent);
+  c->AsT = ar.alloc<double>(4L * F.p2.sell.nent);
   c->topv = ar.alloc<double>(N1);
   c->mvec = ar.alloc<double>(N1);
   c->arhs = ar.alloc<double>(nmax);
@@ -2098,9 +2085,7 @@ chnss_status adjoint_step(chnss_ctx *c, const chnss_state *stk, const chnss_stat
   // transposed fine operators
   sell_gather_transposed(F.p1.sell, 1, c->L[0], c->LsT, s);
   sell_gather_transposed(F.p1.sell, 1, c->AC[0], c->ACsT, s);
-  // the symmetric gradient's off-diagonal entries serve both orders
-  if (c->p2fine()) p2_values<double>(F, m.top_bc, c->A[0], true, c->AsT, nullptr, s);
-  else sell_gather_transposed(F.p2.sell, 4, c->A[0], c->AsT, s);
+  sell_gather_transposed(F.p2.sell, 4, c->A[0], c->AsT, s);
   for (int k = 0; k < 3; ++k) vec_fill(N1, 0.0, out->phi[k], s);
   for (int k = 0; k < 4; ++k) vec_fill(N1, 0.0, out->mu[k], s);
   vec_fill(N1, 0.0, out->Phi_v, s);

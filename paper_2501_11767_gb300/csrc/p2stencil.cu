@@ -8,33 +8,7 @@ constexpr int TPB = 256;
 
 constexpr SlotTable kSlots = slot_table();
 
-// slot of the row of slot k's column that points back (its transposed entry)
-constexpr int back_slot(int ty, int k) {
-  const int di = kSlots.di[slot_base(ty) + k], dj = kSlots.dj[slot_base(ty) + k];
-  const int tc = type_of((ty & 1) + (di & 1), (ty >> 1) + (dj & 1));
-  for (int q = 0; q < slot_count(tc); ++q)
-    if (kSlots.di[slot_base(tc) + q] == -di && kSlots.dj[slot_base(tc) + q] == -dj) return q;
-  return -1;
-}
-struct BackTable {
-  signed char k[kP2Slots];
-};
-constexpr BackTable make_back() {
-  BackTable b{};
-  for (int ty = 0; ty < 4; ++ty)
-    for (int k = 0; k < slot_count(ty); ++k) b.k[slot_base(ty) + k] = (signed char)back_slot(ty, k);
-  return b;
-}
-constexpr BackTable kBack = make_back();
-constexpr bool back_complete() {
-  for (int k = 0; k < kP2Slots; ++k)
-    if (kBack.k[k] < 0) return false;
-  return true;
-}
-static_assert(back_complete(), "the stencil is structurally symmetric");
-
 __constant__ SlotTable c_slots = kSlots;
-__constant__ BackTable c_back = kBack;
 
 template <typename T> struct V2;
 template <> struct V2<float> { using type = float2; };
@@ -98,8 +72,8 @@ struct NodeIn {
 // Fine levels: one cell (its four nodes) a thread.  The 19 neighbours of the
 // vertex are all the cell reads, every value load is one coalesced access of
 // two values, and all loads are independent.
-template <typename T, typename VT, bool OPEN, bool VEC>
-__global__ void __launch_bounds__(kSellMaxBlock, sizeof(T) == 4 ? 2 : 1) k_p2_spmv(int n, long ld, const VT *__restrict__ val,
+template <typename T, typename VT, bool OPEN>
+__global__ void __launch_bounds__(kSellMaxBlock, 2) k_p2_spmv(int n, long ld, const VT *__restrict__ val,
                                                            const T *__restrict__ u, T *out, int mode, int start,
                                                            Args a, const __grid_constant__ Coef<T> cf) {
   using P = typename V2<T>::type;
@@ -114,8 +88,7 @@ __global__ void __launch_bounds__(kSellMaxBlock, sizeof(T) == 4 ? 2 : 1) k_p2_sp
       const P d = static_cast<const P *>(a.dinv)[r], b = static_cast<const P *>(a.b)[r];
       return mk<T>(sc * d.x * b.x, sc * d.y * b.y);
     }
-    if (VEC) return reinterpret_cast<const P *>(u)[r];
-    return mk<T>(u[2 * r], u[2 * r + 1]);
+    return reinterpret_cast<const P *>(u)[r];
   };
   const long r0 = (long)(2 * j) * m + 2 * i;
   constexpr SlotTable st = slot_table();
@@ -231,9 +204,9 @@ __global__ void __launch_bounds__(32 * KS) k_p2_split(int n, long ld, const VT *
 // diagonal values of every block, slot by slot; entry k of a row is its k-th
 // CSR entry (rows with prescribed velocity have none, an open top's rows lack
 // the last ones)
-template <typename VT, bool TRANS>
+template <typename VT>
 __global__ void k_p2_values(int n, int open, long ld, const int *__restrict__ rowptr, const double *__restrict__ A,
-                            VT *__restrict__ out, double *__restrict__ out2) {
+                            VT *__restrict__ out) {
   const int cell = blockIdx.x * TPB + threadIdx.x, k = blockIdx.y;
   if (cell >= ld) return;
   const int w1 = n + 1, m = 2 * n + 1, j = cell / w1, i = cell - j * w1;
@@ -242,14 +215,12 @@ __global__ void k_p2_values(int n, int open, long ld, const int *__restrict__ ro
   const int CI = I + c_slots.di[k], CJ = J + c_slots.dj[k];
   double2 v = make_double2(0.0, 0.0);
   if (cell < w1 * w1 && !prescribed(I, J, m, open) && !prescribed(CI, CJ, m, open)) {
-    const int r = TRANS ? CJ * m + CI : J * m + I;
-    const int q = rowptr[r] + (TRANS ? c_back.k[k] : k - slot_base(ty));
+    const int q = rowptr[J * m + I] + k - slot_base(ty);
     v = make_double2(A[4L * q], A[4L * q + 3]);
   }
   const long e = 2 * (k * ld + cell);
   out[e] = from_double<VT>(v.x);
   out[e + 1] = from_double<VT>(v.y);
-  if (out2) *reinterpret_cast<double2 *>(out2 + e) = v;
 }
 
 // the off-diagonal entries of the rows nearest the centre, then a check of
@@ -329,23 +300,20 @@ P2Table p2_table(Arena &keep, const Level &L, int open_top, const double *A, cud
   t.ok = hbad == 0;
   std::vector<float> f(t.c, t.c + kCount), h(kCount);
   for (int k = 0; k < kCount; ++k) h[k] = __bfloat162float(__double2bfloat16(t.c[k]));
-  t.d64 = keep.upload(std::vector<double>(t.c, t.c + kCount));
   t.d32 = keep.upload(f);
   t.d16 = keep.upload(h);
   return t;
 }
 
 template <typename VT>
-void p2_values(const Level &L, int open_top, const double *A, bool transposed, VT *out, double *out2, cudaStream_t s) {
+void p2_values(const Level &L, int open_top, const double *A, VT *out, cudaStream_t s) {
   const long ld = p2_ld(L.n);
   const dim3 g((unsigned)((ld + TPB - 1) / TPB), kP2Slots);
-  if (transposed) k_p2_values<VT, true><<<g, TPB, 0, s>>>(L.n, open_top, ld, L.p2.rowptr, A, out, out2);
-  else k_p2_values<VT, false><<<g, TPB, 0, s>>>(L.n, open_top, ld, L.p2.rowptr, A, out, out2);
+  k_p2_values<VT><<<g, TPB, 0, s>>>(L.n, open_top, ld, L.p2.rowptr, A, out);
   CHNSS_LAUNCH_CK();
 }
-template void p2_values<float>(const Level &, int, const double *, bool, float *, double *, cudaStream_t);
-template void p2_values<double>(const Level &, int, const double *, bool, double *, double *, cudaStream_t);
-template void p2_values<__nv_bfloat16>(const Level &, int, const double *, bool, __nv_bfloat16 *, double *, cudaStream_t);
+template void p2_values<float>(const Level &, int, const double *, float *, cudaStream_t);
+template void p2_values<__nv_bfloat16>(const Level &, int, const double *, __nv_bfloat16 *, cudaStream_t);
 
 namespace {
 inline bool aligned(const void *p, size_t bytes) { return (reinterpret_cast<uintptr_t>(p) % bytes) == 0; }
@@ -355,29 +323,18 @@ void launch(const Level &L, int ks, const VT *val, const T *u, T *out, SpmvMode 
             const Coef<T> &cf, const T *tab, cudaStream_t s) {
   const int cells = (L.n + 1) * (L.n + 1), tpb = L.p2.sell.block, nb = (cells + tpb - 1) / tpb;
   const long ld = p2_ld(L.n);
-  if (!aligned(u, 2 * sizeof(T))) {   // a caller's solution vector
-    if constexpr (sizeof(T) == 8) {
-      k_p2_spmv<T, VT, OPEN, false><<<nb, tpb, 0, s>>>(L.n, ld, val, u, out, mode, start, a, cf);
-      return;
-    }
-    throw Error{CHNSS_ERR_ARG, "velocity vectors must be aligned to one node"};
+  const dim3 gs((unsigned)((cells + 31) / 32), 4);
+  switch (ks) {
+    case 2: k_p2_split<VT, 2, OPEN><<<gs, 64, 0, s>>>(L.n, ld, val, u, out, mode, start, a, tab); return;
+    case 4: k_p2_split<VT, 4, OPEN><<<gs, 128, 0, s>>>(L.n, ld, val, u, out, mode, start, a, tab); return;
+    case 8: k_p2_split<VT, 8, OPEN><<<gs, 256, 0, s>>>(L.n, ld, val, u, out, mode, start, a, tab); return;
   }
-  if constexpr (sizeof(T) == 4) {
-    const dim3 gs((unsigned)((cells + 31) / 32), 4);
-    switch (ks) {
-      case 2: k_p2_split<VT, 2, OPEN><<<gs, 64, 0, s>>>(L.n, ld, val, u, out, mode, start, a, tab); return;
-      case 4: k_p2_split<VT, 4, OPEN><<<gs, 128, 0, s>>>(L.n, ld, val, u, out, mode, start, a, tab); return;
-      case 8: k_p2_split<VT, 8, OPEN><<<gs, 256, 0, s>>>(L.n, ld, val, u, out, mode, start, a, tab); return;
-    }
-  }
-  k_p2_spmv<T, VT, OPEN, true><<<nb, tpb, 0, s>>>(L.n, ld, val, u, out, mode, start, a, cf);
+  k_p2_spmv<T, VT, OPEN><<<nb, tpb, 0, s>>>(L.n, ld, val, u, out, mode, start, a, cf);
 }
 // the table in the precision of the values, on the device and (rounded the
 // same way) as kernel arguments
-const double *device_table(const P2Table &t, const double *) { return t.d64; }
 const float *device_table(const P2Table &t, const float *) { return t.d32; }
 const float *device_table(const P2Table &t, const __nv_bfloat16 *) { return t.d16; }
-double rounded(double x, const double *) { return x; }
 float rounded(double x, const float *) { return (float)x; }
 float rounded(double x, const __nv_bfloat16 *) { return __bfloat162float(__double2bfloat16(x)); }
 }  // namespace
@@ -471,10 +428,11 @@ template void p2_restrict<double>(int, int, const double *, double *, cudaStream
 template void p2_prolong_add<float>(int, int, const float *, float *, cudaStream_t);
 template void p2_prolong_add<double>(int, int, const double *, double *, cudaStream_t);
 
-template <typename T, typename VT>
-void p2_spmv(const Level &L, int open_top, const P2Table &tab, const VT *val, const T *u, T *out, SpmvMode mode,
+template <typename VT>
+void p2_spmv(const Level &L, int open_top, const P2Table &tab, const VT *val, const float *u, float *out, SpmvMode mode,
              const SpmvArgs &a, P2Start start, const double *scale, cudaStream_t s) {
-  for (const void *q : {(const void *)out, a.b, a.w, a.dinv})
+  using T = float;
+  for (const void *q : {(const void *)u, (const void *)out, a.b, a.w, a.dinv})
     if (!aligned(q, 2 * sizeof(T))) throw Error{CHNSS_ERR_ARG, "velocity vectors must be aligned to one node"};
   Coef<T> cf;
   for (int k = 0; k < kCount; ++k) cf.c[k] = rounded(tab.c[k], val);
@@ -485,11 +443,9 @@ void p2_spmv(const Level &L, int open_top, const P2Table &tab, const VT *val, co
   else launch<T, VT, false>(L, ks, val, u, out, mode, start, ka, cf, dt, s);
   CHNSS_LAUNCH_CK();
 }
-template void p2_spmv<float, float>(const Level &, int, const P2Table &, const float *, const float *, float *,
+template void p2_spmv<float>(const Level &, int, const P2Table &, const float *, const float *, float *,
                                     SpmvMode, const SpmvArgs &, P2Start, const double *, cudaStream_t);
-template void p2_spmv<float, __nv_bfloat16>(const Level &, int, const P2Table &, const __nv_bfloat16 *, const float *,
+template void p2_spmv<__nv_bfloat16>(const Level &, int, const P2Table &, const __nv_bfloat16 *, const float *,
                                             float *, SpmvMode, const SpmvArgs &, P2Start, const double *, cudaStream_t);
-template void p2_spmv<double, double>(const Level &, int, const P2Table &, const double *, const double *, double *,
-                                      SpmvMode, const SpmvArgs &, P2Start, const double *, cudaStream_t);
 
 }  // namespace chnss

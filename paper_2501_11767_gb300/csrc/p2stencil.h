@@ -24,8 +24,7 @@ constexpr int kP2TopSlots = 28;                  // vertex and horizontal slots 
 // off-diagonal entries (0,1) and (1,0) by slot; rows on an open top from kP2Slots on
 struct P2Table {
   double c[2 * (kP2Slots + kP2TopSlots)];
-  // device copies: FP64, rounded to FP32, rounded to BF16 (as FP32)
-  const double *d64 = nullptr;
+  // device copies: rounded to FP32, rounded to BF16 (as FP32)
   const float *d32 = nullptr, *d16 = nullptr;
   bool ok = false;                               // every row of the level matches it
 };
@@ -44,10 +43,9 @@ bool p2_applies(const Level &L, const P2Table &t, size_t value_size);
 // Table of the level's constant blocks A (CSR order, 4 values each) and
 // whether all its rows match it (synchronises s); device copies from keep.
 P2Table p2_table(Arena &keep, const Level &L, int open_top, const double *A, cudaStream_t s);
-// Diagonal values of A (or of its transpose) in stencil order; out2 (may be
-// null) receives a second copy in FP64
+// Diagonal values of A in stencil order
 template <typename VT>
-void p2_values(const Level &L, int open_top, const double *A, bool transposed, VT *out, double *out2, cudaStream_t s);
+void p2_values(const Level &L, int open_top, const double *A, VT *out, cudaStream_t s);
 
 // How a Chebyshev sweep (SPMV_CHEB) takes its previous iterates:
 //   P2_PLAIN  u from u, w from args.w (or none)
@@ -56,8 +54,8 @@ void p2_values(const Level &L, int open_top, const double *A, bool transposed, V
 enum P2Start { P2_PLAIN = 0, P2_FIRST = 1, P2_SECOND = 2 };
 
 // Same row sums, in the same order, as spmv_sell_bsr2 on the level's pattern.
-template <typename T, typename VT>
-void p2_spmv(const Level &L, int open_top, const P2Table &tab, const VT *val, const T *u, T *out, SpmvMode mode,
+template <typename VT>
+void p2_spmv(const Level &L, int open_top, const P2Table &tab, const VT *val, const float *u, float *out, SpmvMode mode,
              const SpmvArgs &a, P2Start start, const double *scale, cudaStream_t s);
 
 // b = R r onto the mesh of nc cells a side; x += P xc from it: quadratic

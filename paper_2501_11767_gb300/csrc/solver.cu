@@ -269,9 +269,9 @@ template <typename T>
 template <typename VT>
 void MGHier<T>::gather_values(int l, VT *out, cudaStream_t s) const {
   if (kind == 2) sell_gather9<VT>(bpat[l]->sell.nent, bmap[l], val64[l], out, s);
-  else if (stencil(l, sizeof(VT)))
-    p2_values<VT>(*p2lev[l], open_top, val64[l], false, out, l == 0 && sizeof(VT) < 8 ? copy64 : nullptr, s);
-  else sell_gather<VT>(pat[l]->sell, kind == 0 ? 1 : 4, val64[l], out, s);
+  else if (stencil(l, sizeof(VT))) {
+    if constexpr (sizeof(VT) < 8) p2_values<VT>(*p2lev[l], open_top, val64[l], out, s);
+  } else sell_gather<VT>(pat[l]->sell, kind == 0 ? 1 : 4, val64[l], out, s);
 }
 
 template <typename T>
@@ -279,7 +279,7 @@ void MGHier<T>::setup(cudaStream_t s) {
   for (int l = 0; l < nl; ++l) {
     if (bf16) gather_values<__nv_bfloat16>(l, val16[l], s);
     else gather_values<T>(l, val[l], s);
-    if (l == 0 && val0_64 && val0_64 != copy64) gather_values<double>(0, val0_64, s);
+    if (l == 0 && val0_64) gather_values<double>(0, val0_64, s);
     if (l == nl - 1 && !coarse_iter) break;
     if (kind == 1)
       jacobi_bsr2<T>(*pat[l], val64[l], diag[l], dinv[l], hi[l], partial, s);
@@ -319,17 +319,12 @@ void MGHier<T>::op(int l, const T *u, T *out, SpmvMode mode, const SpmvArgs &a, 
 template <typename T>
 void MGHier<T>::spmv_level(int l, const T *u, T *out, SpmvMode mode, const SpmvArgs &a, cudaStream_t s,
                            P2Start start) {
-  if (stencil(l)) {
-    if constexpr (std::is_same<T, float>::value) {
-      if (bf16) {
-        p2_spmv<float, __nv_bfloat16>(*p2lev[l], open_top, p2tab[l], val16[l], u, out, mode, a, start, coef[l], s);
-        return;
-      }
-    }
-    p2_spmv<T, T>(*p2lev[l], open_top, p2tab[l], val[l], u, out, mode, a, start, coef[l], s);
-    return;
-  }
   if constexpr (std::is_same<T, float>::value) {
+    if (stencil(l)) {
+      if (bf16) p2_spmv<__nv_bfloat16>(*p2lev[l], open_top, p2tab[l], val16[l], u, out, mode, a, start, coef[l], s);
+      else p2_spmv<float>(*p2lev[l], open_top, p2tab[l], val[l], u, out, mode, a, start, coef[l], s);
+      return;
+    }
     if (bf16) {
       if (kind == 0) spmv_sell(*pat[l], val16[l], 1, u, out, mode, a, s);
       else if (kind == 1) spmv_sell_bsr2(*pat[l], val16[l], u, out, mode, a, s);
@@ -494,7 +489,7 @@ void MGHier<T>::enable_inner(Arena &ar, double rtol, int maxit, cudaStream_t bod
   acc = ar.alloc<double>(n[0]);
   if (!std::is_same<T, double>::value) {
     r64 = ar.alloc<double>(n[0]);
-    val0_64 = copy64 ? copy64 : ar.alloc<double>(sell_values(0, sizeof(double)));
+    val0_64 = ar.alloc<double>(sell_values(0, sizeof(double)));
   }
   ictl = ar.alloc<double>(8);
   iit = ar.alloc<int>(1);
@@ -536,8 +531,6 @@ void MGHier<T>::inner_residual(cudaStream_t s) {
     dot<double>(n[0], b[0], b[0], ictl + 1, ipartial, s);
   } else {
     if (kind == 0) spmv_sell<double>(*pat[0], val0_64, 1, acc, r64, SPMV_RES, a, s);
-    else if (stencil(0, sizeof(double)))
-      p2_spmv<double, double>(*p2lev[0], open_top, p2tab[0], val0_64, acc, r64, SPMV_RES, a, P2_PLAIN, nullptr, s);
     else if (kind == 1) spmv_sell_bsr2<double>(*pat[0], val0_64, acc, r64, SPMV_RES, a, s);
     else spmv_sell_bsr3<double>(*bpat[0], val0_64, acc, r64, SPMV_RES, a, s);
     dot<double>(n[0], r64, r64, ictl + 1, ipartial, s);

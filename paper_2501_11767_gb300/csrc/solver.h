@@ -80,9 +80,6 @@ struct MGHier {
   std::vector<const Level *> p2lev;
   std::vector<P2Table> p2tab;
   int open_top = 0;
-  // level-0 values in FP64 and stencil order, written by setup with the
-  // level's own (T != double; null: not wanted)
-  double *copy64 = nullptr;
   VlcPlan vlc;             // coarse end of the FP32 velocity cycle by one cluster
   bool stencil(int l, size_t value_size) const {
     return kind == 1 && !p2tab.empty() && p2_applies(*p2lev[l], p2tab[l], value_size);
