@@ -427,9 +427,15 @@ chnss_status chnss3_ctx_destroy(chnss3_ctx_t ctx);
 chnss_status chnss3_sizes(chnss3_ctx_t ctx, int *N1, int *N2);
 chnss_status chnss3_step(chnss3_ctx_t ctx, const chnss_state *in, chnss_state *out, chnss_solve_info *info);
 /* on != 0 (default): the three solve groups (CH species then the air
- * potential; AC; Oseen) of chnss3_step run concurrently on library streams;
- * 0: one after the other.  Results are bitwise the same. */
+ * potential; AC; Oseen) of chnss3_step run concurrently on library streams
+ * and the independent parts of a preconditioner are parallel graph branches;
+ * 0: one after the other, one kernel at a time.  Results are bitwise the
+ * same.  Changing the setting drops the captured preconditioners (captured
+ * again at their next use). */
 chnss_status chnss3_set_step_concurrency(chnss3_ctx_t ctx, int on);
+/* For tests: parallel branches of the captured graph of preconditioner prec
+ * (0..2 CH species, 3 AC, 4 Oseen; 1: one kernel at a time); 0: not captured. */
+chnss_status chnss3_debug_prec_branches(chnss3_ctx_t ctx, int prec, int *branches);
 const char *chnss3_last_error(chnss3_ctx_t ctx);
 /* Adjoint of one 3D step: the discrete adjoint of chnss3_step, with the
  * same contributions as chnss_adjoint_step (transposed solves by FGMRES to a

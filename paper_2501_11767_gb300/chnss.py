@@ -153,6 +153,7 @@ EXPORTS = {
                                    ctypes.POINTER(SolveInfo)]),
     "chnss3_last_error": (ctypes.c_char_p, [ctypes.c_void_p]),
     "chnss3_set_step_concurrency": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int]),
+    "chnss3_debug_prec_branches": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.POINTER(ctypes.c_int)]),
     "chnss3_adjoint_step": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(State), ctypes.POINTER(State),
                                            ctypes.POINTER(State), ctypes.POINTER(State),
                                            ctypes.POINTER(ctypes.c_double), ctypes.POINTER(SolveInfo)]),
@@ -496,6 +497,12 @@ class Context3:
 
     def set_step_concurrency(self, on: bool):
         _check(load().chnss3_set_step_concurrency(self._h, 1 if on else 0))
+
+    def debug_prec_branches(self, prec: int) -> int:
+        """chnss3_debug_prec_branches: branches of a captured preconditioner."""
+        out = ctypes.c_int()
+        self._check3(load().chnss3_debug_prec_branches(self._h, prec, ctypes.byref(out)))
+        return out.value
 
     def new_state(self):
         import torch

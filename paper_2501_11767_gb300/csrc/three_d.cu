@@ -956,7 +956,9 @@ struct chnss3_ctx {
   // captured preconditioners (0..2 CH species, 3 AC, 4 Oseen) replayed from
   // fixed staging vectors; each captured on a private stream of its own
   cudaStream_t cap[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-  // their side branches (independent parts of one preconditioner)
+  // their side branches (independent parts of one preconditioner; none when
+  // concurrent is off); branches of each captured graph
+  int branches[5] = {};
   cudaStream_t side[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
   cudaEvent_t ev_fork[5] = {}, ev_join[5] = {};
   // bodies of the inner multigrid loops (inner_rtol > 0), one stream per solve group
@@ -1487,13 +1489,15 @@ void mg_apply(MGHier<T> &h, long n, const double *r, double *z, cudaStream_t s) 
 
 // Side branch of preconditioner g's graph, forked off s and joined back
 // (s is capturing: its levels are latency bound, so independent V-cycles run
-// beside each other).
+// beside each other).  Without concurrency the "side" is s itself.
 cudaStream_t fork3(chnss3_ctx *c, int g, cudaStream_t s) {
+  if (!c->concurrent) return s;
   CHNSS_CK(cudaEventRecord(c->ev_fork[g], s));
   CHNSS_CK(cudaStreamWaitEvent(c->side[g], c->ev_fork[g], 0));
   return c->side[g];
 }
 void join3(chnss3_ctx *c, int g, cudaStream_t s) {
+  if (!c->concurrent) return;
   CHNSS_CK(cudaEventRecord(c->ev_join[g], c->side[g]));
   CHNSS_CK(cudaStreamWaitEvent(s, c->ev_join[g], 0));
 }
@@ -1553,6 +1557,21 @@ void prec_body3(chnss3_ctx *c, int g, const double *r, double *z, cudaStream_t s
   }
 }
 
+// parallel branches of a graph: its roots, and every successor of a node
+// beyond the first (1: one kernel at a time)
+int graph_branches(cudaGraph_t graph) {
+  size_t n = 0, roots = 0;
+  CHNSS_CK(cudaGraphGetRootNodes(graph, nullptr, &roots));
+  CHNSS_CK(cudaGraphGetEdges(graph, nullptr, nullptr, nullptr, &n));
+  std::vector<cudaGraphNode_t> from(n), to(n);
+  std::vector<cudaGraphEdgeData> data(n);
+  if (n > 0) CHNSS_CK(cudaGraphGetEdges(graph, from.data(), to.data(), data.data(), &n));
+  std::sort(from.begin(), from.end());
+  int branches = (int)roots;
+  for (size_t i = 1; i < n; ++i) branches += from[i] == from[i - 1];
+  return branches;
+}
+
 // z = P_g r through the captured graph of preconditioner g (captured at the
 // first application; the hierarchies' values change in place between steps)
 void run_prec3(chnss3_ctx *c, int g, long n, const double *r, double *z, cudaStream_t s) {
@@ -1568,6 +1587,7 @@ void run_prec3(chnss3_ctx *c, int g, long n, const double *r, double *z, cudaStr
       throw;
     }
     CHNSS_CK(cudaStreamEndCapture(c->cap[g], &graph));
+    c->branches[g] = graph_branches(graph);
     const cudaError_t e = cudaGraphInstantiate(&c->gexec[g], graph, 0);
     cudaGraphDestroy(graph);
     CHNSS_CK(e);
@@ -2161,7 +2181,33 @@ extern "C" chnss_status chnss3_set_step_concurrency(chnss3_ctx_t ctx, int on) {
     chnss::set_global_error("null context");
     return CHNSS_ERR_ARG;
   }
-  ctx->concurrent = on != 0;
+  using namespace chnss;
+  try {
+    if (ctx->concurrent != (on != 0)) {
+      CHNSS_CK(cudaStreamSynchronize(ctx->s));
+      ctx->concurrent = on != 0;
+      for (cudaGraphExec_t &g : ctx->gexec) {   // their branches follow the setting: captured again at the next use
+        if (g) cudaGraphExecDestroy(g);
+        g = nullptr;
+      }
+    }
+    return CHNSS_OK;
+  } catch (const Error &e) {
+    ctx->err = e.msg;
+    return e.status;
+  }
+}
+
+extern "C" chnss_status chnss3_debug_prec_branches(chnss3_ctx_t ctx, int prec, int *branches) {
+  if (!ctx) {
+    chnss::set_global_error("null context");
+    return CHNSS_ERR_ARG;
+  }
+  if (prec < 0 || prec >= 5 || !branches) {
+    ctx->err = "prec must be 0..4 and branches not null";
+    return CHNSS_ERR_ARG;
+  }
+  *branches = ctx->gexec[prec] ? ctx->branches[prec] : 0;
   return CHNSS_OK;
 }
 
