@@ -308,6 +308,22 @@ chnss_status chnss_debug_cgs2(int arith, long n, int k, const double *V, long ld
 chnss_status chnss_debug_spmv(int layout, int precision, int mode, int nrows, int ncols, const int *rowptr,
                               const int *col, const double *val, const double *x, const double *b, const double *w,
                               const double *dinv, const double *coef, double *y, int *warps_per_slice);
+/* Test entry: whether the device has a place for a cluster of ctas blocks of
+ * the dense-inverse kernel with these threads and bytes of shared memory (a
+ * query; where it is no, contexts are made without such clusters). */
+chnss_status chnss_debug_cluster_runs(int ctas, int threads, long smem, int *runs);
+/* Test entry: one multigrid V-cycle on a block of an assembled context, by a
+ * hierarchy made and set up for the call.  block 0: M + tau C; 1: the
+ * velocity block A; 2: K_p.  precision 0: FP64; 1: FP32; 2 (velocity only):
+ * BF16 values.  clusters 0: no thread-block clusters, as on a device that
+ * has no place for them; 1: as the preconditioners have it (the result is
+ * the same bit for bit).  nvec 0: the single-vector cycle; 1..3 (block 0
+ * only): the multi-vector one.  HOST arrays in, out of max(nvec, 1) vectors.
+ * info[4]: first level that a cluster takes (-1: none), first level of the
+ * one-block tail (-1: none), the dense inverse by a cluster (-1: there is
+ * none), levels swept as a P2 stencil.  Allocates and synchronises. */
+chnss_status chnss_debug_vcycle(chnss_ctx_t ctx, int block, int precision, int clusters, int nvec, const double *in,
+                                double *out, int *info);
 /* Assembled right-hand side of a system (host, chnss_system_size doubles). */
 chnss_status chnss_export_rhs(chnss_ctx_t ctx, chnss_system sys, double *host_out);
 

@@ -140,6 +140,9 @@ EXPORTS = {
                                         ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
                                         ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
                                         ctypes.c_void_p, ctypes.POINTER(ctypes.c_int)]),
+    "chnss_debug_cluster_runs": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_long,
+                                                ctypes.POINTER(ctypes.c_int)]),
+    "chnss_debug_vcycle": (ctypes.c_int, [ctypes.c_void_p] + [ctypes.c_int] * 4 + [ctypes.c_void_p] * 3),
     "chnss_profile_enable": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int]),
     "chnss_profile_read": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(Profile)]),
     "chnss_inner_stats_read": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.POINTER(InnerStats)]),
@@ -466,6 +469,18 @@ class Context:
         _check(load().chnss_inner_stats_read(self._h, 1 if reset else 0, ctypes.byref(st)), self._h)
         return st.as_dict()
 
+    def debug_vcycle(self, block: int, precision: int, clusters: bool, x, nvec: int = 0):
+        """chnss_debug_vcycle: (result, first cluster level, first level of the
+        one-block tail, inverse by a cluster, P2 stencil levels)."""
+        x = np.ascontiguousarray(x, dtype=np.float64)
+        size = max(nvec, 1) * (2 * self.mesh.N2 if block == 1 else self.mesh.N1)
+        if x.size != size:
+            raise ValueError(f"x must hold {size} values")
+        out, info = np.zeros_like(x), np.zeros(4, dtype=np.int32)
+        _check(load().chnss_debug_vcycle(self._h, block, precision, 1 if clusters else 0, nvec, x.ctypes.data,
+                                         out.ctypes.data, info.ctypes.data), self._h)
+        return (out, *info.tolist())
+
     def export_rhs(self, sys: int):
         out = np.zeros(self.system_size(sys), dtype=np.float64)
         _check(load().chnss_export_rhs(self._h, sys, out.ctypes.data), self._h)
@@ -601,6 +616,13 @@ def debug_spmv(layout: int, precision: int, mode: int, rowptr, col, val, x, b=No
                                    val.ctypes.data, x.ctypes.data, ptr(b), ptr(w), ptr(dinv), ptr(coef),
                                    y.ctypes.data, ctypes.byref(k)))
     return y, k.value
+
+
+def debug_cluster_runs(ctas: int, threads: int, smem: int) -> bool:
+    """chnss_debug_cluster_runs: whether the device has a place for the cluster."""
+    out = ctypes.c_int()
+    _check(load().chnss_debug_cluster_runs(ctas, threads, smem, ctypes.byref(out)))
+    return out.value != 0
 
 
 def debug_cgs2(V, w, arith: int):

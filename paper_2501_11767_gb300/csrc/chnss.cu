@@ -560,18 +560,46 @@ void capture_graphs(chnss_ctx *c) {
 }
 
 // ---------------------------------------------------------------------------
+// Multigrid hierarchies of a context's blocks, as its preconditioners have them
+enum Block { BLOCK_CH = 0, BLOCK_VELOCITY = 1, BLOCK_KP = 2 };   // M + tau C, A, K_p
+template <typename T>
+void init_block(chnss_ctx *c, Block block, Arena &ar, MGHier<T> &h) {
+  const bool vel = block == BLOCK_VELOCITY, open = c->mesh->m.top_bc == 1;
+  const std::vector<double *> &src = vel ? c->A : block == BLOCK_CH ? c->L : open ? c->Kpd : c->K1;
+  std::vector<const Pattern *> pats;
+  std::vector<const int *> diags;
+  std::vector<const Transfer *> trs;
+  for (int l = 0; l < c->nlev; ++l) {
+    const Level &L = c->lv(l);
+    pats.push_back(vel ? &L.p2 : &L.p1);
+    diags.push_back(vel ? L.diag2 : L.diag1);
+    if (vel) h.p2lev.push_back(&L);
+    else trs.push_back(&L.t1);
+  }
+  if (vel) {
+    h.p2tab = c->p2tab;
+    h.open_top = c->mesh->m.top_bc;
+    h.degree = 4;        // velocity smoothing: degree 4 on [hi / 16, hi]
+    h.ratio = 16.0;
+  }
+  h.keep_dense = block == BLOCK_KP;   // a pure Laplacian: its coarsest level is not mass-dominated
+  // open top: Dirichlet outflow rows, K_p non-singular.  The CH / AC
+  // hierarchies reduce into partial_ch, the Oseen ones into partial: the two
+  // groups assemble and solve on different streams
+  h.init(ar, vel ? 1 : 0, block == BLOCK_KP && !open, pats, diags, {src.begin(), src.end()}, trs,
+         block == BLOCK_CH ? c->partial_ch : c->partial);
+}
+
 template <typename T>
 void init_precset(chnss_ctx *c, PrecSet<T> &P) {
   Arena &ar = c->ar;
   const int nl = c->nlev;
-  std::vector<const Pattern *> p1s, p2s;
-  std::vector<const int *> d1s, d2s;
+  std::vector<const Pattern *> p1s;
+  std::vector<const int *> d1s;
   std::vector<const Transfer *> t1s;
   for (int l = 0; l < nl; ++l) {
     p1s.push_back(&c->lv(l).p1);
-    p2s.push_back(&c->lv(l).p2);
     d1s.push_back(c->lv(l).diag1);
-    d2s.push_back(c->lv(l).diag2);
     t1s.push_back(&c->lv(l).t1);
   }
   auto vals = [&](const std::vector<double *> &v) { return std::vector<const double *>(v.begin(), v.end()); };
@@ -579,9 +607,7 @@ void init_precset(chnss_ctx *c, PrecSet<T> &P) {
   // dominant SpMV stream by 40 %.  (The P1 hierarchies save only 25 % per
   // entry and cost more CH iterations than they save: 39 -> 48 at 1024^2.)
   P.A.bf16 = c->p.precision == 2;
-  // the CH / AC hierarchies reduce into partial_ch, the Oseen ones into
-  // partial: the two groups assemble and solve on different streams
-  P.L.init(ar, 0, false, p1s, d1s, vals(c->L), t1s, c->partial_ch);
+  init_block(c, BLOCK_CH, ar, P.L);
   if (c->p.amg == 1) {
     // the paper's algebraic multigrid for the AC block (Sec. 5): smoothed
     // aggregation of the fine AC matrix, its levels set up again every step
@@ -596,18 +622,9 @@ void init_precset(chnss_ctx *c, PrecSet<T> &P) {
   } else {
     P.AC.init(ar, 0, false, p1s, d1s, vals(c->AC), t1s, c->partial_ch);
   }
-  for (int l = 0; l < nl; ++l) P.A.p2lev.push_back(&c->lv(l));
-  P.A.p2tab = c->p2tab;
-  P.A.open_top = c->mesh->m.top_bc;
-  P.A.degree = 4;        // velocity smoothing: degree 4 on [hi / 16, hi]
-  P.A.ratio = 16.0;
-  P.A.init(ar, 1, false, p2s, d2s, vals(c->A), {}, c->partial);   // transfers: p2lev
+  init_block(c, BLOCK_VELOCITY, ar, P.A);
   c->As = ar.alloc<double>(4L * c->lv(0).p2.sell.nent);   // the fine operator applied inside FGMRES
-  P.Kp.keep_dense = true;       // a pure Laplacian: its coarsest level is not mass-dominated
-  if (c->mesh->m.top_bc == 1)   // open top: Dirichlet outflow rows, non-singular
-    P.Kp.init(ar, 0, false, p1s, d1s, vals(c->Kpd), t1s, c->partial);
-  else
-    P.Kp.init(ar, 0, true, p1s, d1s, vals(c->K1), t1s, c->partial);
+  init_block(c, BLOCK_KP, ar, P.Kp);
   for (int sp = 0; sp < 3; ++sp) {
     std::vector<const double *> x1, x2;
     for (int l = 0; l < nl; ++l) {
@@ -1513,6 +1530,43 @@ void debug_spmv_run(int layout, int mode, Pattern &P, const std::vector<int> &hm
 }
 
 }  // namespace debug_spmv_detail
+
+namespace debug_vcycle_detail {
+
+// One V-cycle of chnss_debug_vcycle on a hierarchy of its own.
+template <typename T>
+void run(chnss_ctx *c, int block, bool bf16, bool clusters, int nvec, const double *in, double *out, int *info) {
+  Arena ar;
+  MGHier<T> h;
+  MGBatch<T> hb;
+  h.bf16 = bf16;
+  h.clusters = clusters;
+  init_block(c, (Block)block, ar, h);
+  cudaStream_t s = c->s;
+  h.setup(s);
+  if (nvec > 0) hb.init(ar, &h, nvec);
+  const long n = h.n[0];
+  std::vector<T> v(n);
+  for (int k = 0; k < std::max(nvec, 1); ++k) {
+    for (long i = 0; i < n; ++i) v[i] = (T)in[k * n + i];
+    CHNSS_CK(cudaMemcpyAsync(nvec > 0 ? hb.input(k) : h.input(), v.data(), n * sizeof(T), cudaMemcpyHostToDevice, s));
+    CHNSS_CK(cudaStreamSynchronize(s));
+  }
+  if (nvec > 0) hb.apply(s);
+  else h.apply(s);
+  for (int k = 0; k < std::max(nvec, 1); ++k) {
+    CHNSS_CK(cudaMemcpyAsync(v.data(), nvec > 0 ? hb.output(k) : h.output(), n * sizeof(T), cudaMemcpyDeviceToHost, s));
+    CHNSS_CK(cudaStreamSynchronize(s));
+    for (long i = 0; i < n; ++i) out[k * n + i] = (double)v[i];
+  }
+  info[0] = nvec > 0 ? hb.mgc.first : block == BLOCK_VELOCITY ? h.vlc.first : h.mgc.first;
+  info[1] = nvec > 0 ? -1 : h.tail_l0;
+  info[2] = h.coarse_iter ? -1 : h.inv_cluster ? 1 : 0;
+  info[3] = 0;
+  for (int l = 0; l < h.nl; ++l) info[3] += h.stencil(l) ? 1 : 0;
+}
+
+}  // namespace debug_vcycle_detail
 }  // namespace chnss
 
 extern "C" {
@@ -1784,6 +1838,31 @@ chnss_status chnss_debug_cgs2(int arith, long n, int k, const double *V, long ld
   ABI_CATCH(nullptr)
 }
 
+
+chnss_status chnss_debug_cluster_runs(int ctas, int threads, long smem, int *runs) {
+  ABI_TRY
+  if (ctas < 1 || threads < 1 || smem < 0 || !runs) throw Error{CHNSS_ERR_ARG, "bad cluster or null argument"};
+  *runs = dense_cluster_runs(ctas, threads, (size_t)smem) ? 1 : 0;
+  return CHNSS_OK;
+  ABI_CATCH(nullptr)
+}
+
+chnss_status chnss_debug_vcycle(chnss_ctx_t ctx, int block, int precision, int clusters, int nvec, const double *in,
+                                double *out, int *info) {
+  if (!ctx) return fail(nullptr, CHNSS_ERR_ARG, "null context");
+  ABI_TRY
+  if (block < 0 || block > 2) throw Error{CHNSS_ERR_ARG, "block must be 0 (M + tau C), 1 (velocity) or 2 (K_p)"};
+  if (precision < 0 || precision > 2 || (precision == 2 && block != 1))
+    throw Error{CHNSS_ERR_ARG, "precision must be 0, 1 or (velocity only) 2"};
+  if (nvec < 0 || nvec > 3 || (nvec > 0 && block != 0))
+    throw Error{CHNSS_ERR_ARG, "nvec must be 0 or (M + tau C only) 1 to 3"};
+  if (!in || !out || !info) throw Error{CHNSS_ERR_ARG, "null argument"};
+  if (!ctx->assembled) throw Error{CHNSS_ERR_STATE, "a V-cycle needs an assembled context"};
+  if (precision == 0) debug_vcycle_detail::run<double>(ctx, block, false, clusters != 0, nvec, in, out, info);
+  else debug_vcycle_detail::run<float>(ctx, block, precision == 2, clusters != 0, nvec, in, out, info);
+  return CHNSS_OK;
+  ABI_CATCH(ctx)
+}
 
 chnss_status chnss_debug_spmv(int layout, int precision, int mode, int nrows, int ncols, const int *rowptr,
                               const int *col, const double *val, const double *x, const double *b, const double *w,

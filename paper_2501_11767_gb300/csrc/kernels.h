@@ -281,11 +281,14 @@ void pcg_start(long n, const double *dinv, const double *b, double *x, double *p
 void pcg_iteration(const Pattern &P, const double *val, const double *dinv, double *x, const double *p_old,
                    double *p_new, int maxit, const PcgWork &w, cudaStream_t s);
 
-// dense coarse-grid inverse (one CTA, Gauss-Jordan with partial pivoting)
+// dense coarse-grid inverse (Gauss-Jordan with partial pivoting)
 void coarse_dense_csr(const Pattern &P, const double *val, double add_all, double *dense, cudaStream_t s);
 void coarse_dense_bsr2(const Pattern &P, const double *val, double *dense, cudaStream_t s);
+// cluster: by one thread-block cluster (only where dense_cluster_runs(n)), otherwise by one block.
 // unit (may be null, n even): nonzero where rows and columns 2 i, 2 i + 1 are the identity's
-void dense_invert(int n, double *a, double *inv, int *status, cudaStream_t s, const int *unit = nullptr);
+bool dense_cluster_runs(int n);
+bool dense_cluster_runs(int ctas, int threads, size_t smem);   // that kernel in a cluster of another shape
+void dense_invert(int n, double *a, double *inv, int *status, cudaStream_t s, bool cluster, const int *unit = nullptr);
 template <typename T>
 void dense_apply(int n, const double *inv, const T *b, T *x, cudaStream_t s);
 

@@ -325,6 +325,17 @@ __global__ void __launch_bounds__(mgc_threads<T>()) k_p1_cluster(const MgcDesc<T
   }
 }
 
+template <typename T>
+bool runs(int nr, int ctas, size_t smem) {
+  constexpr size_t most = kSmemLimit - sizeof(MgcDesc<T>);
+  switch (nr) {
+    case 1: return cluster_runs<k_p1_cluster<T, 1>>(ctas, mgc_threads<T>(), smem, most);
+    case 2: return cluster_runs<k_p1_cluster<T, 2>>(ctas, mgc_threads<T>(), smem, most);
+    case 3: return cluster_runs<k_p1_cluster<T, 3>>(ctas, mgc_threads<T>(), smem, most);
+    default: return false;
+  }
+}
+
 }  // namespace
 
 template <typename T>
@@ -403,7 +414,7 @@ MgcPlan<T> mgc_plan(Arena &ar, int nr, const std::vector<const Pattern *> &pats,
       d.r_off = take(nr * d.r_vec);
     }
     const size_t bytes = (size_t)off * sizeof(T);
-    if (!ok || bytes > kSmemLimit - sizeof(MgcDesc<T>)) continue;
+    if (!ok || bytes > kSmemLimit - sizeof(MgcDesc<T>) || !runs<T>(nr, plan.ctas, bytes)) continue;
     for (int k = 0; k < nr; ++k) {
       d.b.p[k] = b[first].p[k];
       d.x.p[k] = x[first].p[k];
@@ -423,15 +434,12 @@ void mgc_apply(const MgcPlan<T> &p, cudaStream_t s) {
   const MgcDesc<T> *d = p.desc;
   switch (p.nr) {
     case 1:
-      allow_cluster<k_p1_cluster<T, 1>>(kSmemLimit - sizeof(MgcDesc<T>));
       launch_cluster(k_p1_cluster<T, 1>, p.ctas, 1, mgc_threads<T>(), p.smem, s, d);
       break;
     case 2:
-      allow_cluster<k_p1_cluster<T, 2>>(kSmemLimit - sizeof(MgcDesc<T>));
       launch_cluster(k_p1_cluster<T, 2>, p.ctas, 1, mgc_threads<T>(), p.smem, s, d);
       break;
     case 3:
-      allow_cluster<k_p1_cluster<T, 3>>(kSmemLimit - sizeof(MgcDesc<T>));
       launch_cluster(k_p1_cluster<T, 3>, p.ctas, 1, mgc_threads<T>(), p.smem, s, d);
       break;
     default: throw Error{CHNSS_ERR_ARG, "coarse-level cluster: 1 to 3 vectors"};

@@ -38,7 +38,8 @@ struct MgcPlan {
 };
 
 // Plan for the coarse end of a hierarchy of stencil levels `pats` (finest
-// first, P1 transfers between them) and nr vectors; first = -1 if none fits.
+// first, P1 transfers between them) and nr vectors; first = -1 if none fits
+// or the device has no place for its cluster.
 // The arrays are those of MGHier / MGBatch.
 template <typename T>
 MgcPlan<T> mgc_plan(Arena &ar, int nr, const std::vector<const Pattern *> &pats, const std::vector<const Transfer *> &trs,

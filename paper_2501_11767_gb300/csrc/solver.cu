@@ -173,11 +173,12 @@ void MGHier<T>::init(Arena &ar, int kind_, bool singular_, const std::vector<con
   status = ar.alloc<int>(1);
   partial = partial_buf;
   sum = ar.alloc<double>(1);
+  inv_cluster = clusters && !coarse_iter && dense_cluster_runs(nc);
   if constexpr (std::is_same<T, float>::value) {
-    if (kind == 1 && !p2tab.empty())
+    if (clusters && kind == 1 && !p2tab.empty())
       vlc = vlc_plan(ar, p2lev, open_top, p2tab, val, val16, dinv, coef, b, x, degree, coarse_iter, nc, cinv);
   }
-  if (kind == 0 && !bf16) {
+  if (clusters && kind == 0 && !bf16) {
     std::vector<MultiPtr<T>> X0(nl), B0(nl);
     for (int l = 0; l < nl; ++l) {
       X0[l].p[0] = x[l];
@@ -298,7 +299,7 @@ void MGHier<T>::setup(cudaStream_t s) {
     coarse_dense_bsr2(*pat[L], val64[L], dense, s);
   else
     coarse_dense_csr(*pat[L], val64[L], singular ? 1.0 : 0.0, dense, s);
-  dense_invert(nc, dense, cinv, status, s, kind == 1 && !p2lev.empty() ? p2lev[L]->bnd2 : nullptr);
+  dense_invert(nc, dense, cinv, status, s, inv_cluster, kind == 1 && !p2lev.empty() ? p2lev[L]->bnd2 : nullptr);
 }
 
 template <typename T>
@@ -634,7 +635,8 @@ void MGBatch<T>::init(Arena &ar, MGHier<T> *hier, int nr_) {
       r[l].p[k] = ar.alloc<T>(h->n[l]);
       b[l].p[k] = ar.alloc<T>(h->n[l]);
     }
-  mgc = mgc_plan<T>(ar, nr, h->pat, h->tr, h->val, h->dinv, h->coef, b, x, h->degree, h->coarse_iter, h->nc, h->cinv);
+  if (h->clusters)
+    mgc = mgc_plan<T>(ar, nr, h->pat, h->tr, h->val, h->dinv, h->coef, b, x, h->degree, h->coarse_iter, h->nc, h->cinv);
 }
 
 template <typename T>

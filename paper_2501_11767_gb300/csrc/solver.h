@@ -89,6 +89,8 @@ struct MGHier {
   int nc = 0;
   bool coarse_iter = false;   // coarsest level by Chebyshev steps (kCoarseDegree), no dense inverse
   bool keep_dense = false;    // set before init: dense coarsest level whatever its size (pressure Laplacian)
+  bool clusters = true;       // set before init: thread-block clusters where the device has a place for them
+  bool inv_cluster = false;   // the dense inverse by a cluster
   double *dense = nullptr, *cinv = nullptr;
   int *status = nullptr;
   double *partial = nullptr, *sum = nullptr;
@@ -102,7 +104,7 @@ struct MGHier {
   double ratio = 4.0;      // smoothing interval [hi / ratio, hi]
   // coarse end in one launch: of a cluster on the structured meshes' P1
   // levels (mgc.first..), otherwise of one block (tail_l0.., at most
-  // kTailRows rows each)
+  // kTailRows rows each); every form gives the same bits
   MgcPlan<T> mgc;
   int tail_l0 = -1;
   int tail_width = 8;            // widest tail row (operators and transfers): 8 or 16

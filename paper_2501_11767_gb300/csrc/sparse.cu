@@ -1329,7 +1329,7 @@ __global__ void __launch_bounds__(kInvThreads) k_dense_invert_cluster(int n, con
 // Gauss-Jordan inverse with partial pivoting of a (n x n, row-major,
 // destroyed) into inv; one CTA.  status = 1 on an exactly zero pivot.  For
 // the sizes above kCoarseDenseMax (the pressure Laplacian's coarsest level,
-// inverted once per context).
+// inverted once per context) and devices without a place for the cluster.
 __global__ void k_dense_invert(int n, double *a, double *inv, int *status) {
   __shared__ int piv;
   __shared__ double sv[TPB];
@@ -2621,10 +2621,15 @@ void coarse_dense_bsr2(const Pattern &P, const double *val, double *dense, cudaS
   k_dense_bsr2<<<P.nrows, 128, 0, s>>>(P.nrows, P.rowptr, P.col, val, dense);
   CHNSS_LAUNCH_CK();
 }
-void dense_invert(int n, double *a, double *inv, int *status, cudaStream_t s, const int *unit) {
-  if (n <= kCoarseDenseMax) {
-    constexpr size_t most = sizeof(InvSmem) + 2 * (kCoarseDenseMax / kInvCtas) * kCoarseDenseMax * sizeof(double);
-    allow_cluster<k_dense_invert_cluster>(most);
+constexpr size_t kInvSmemMost = sizeof(InvSmem) + 2 * (kCoarseDenseMax / kInvCtas) * kCoarseDenseMax * sizeof(double);
+bool dense_cluster_runs(int ctas, int threads, size_t smem) {
+  return cluster_runs<k_dense_invert_cluster>(ctas, threads, smem, kInvSmemMost);
+}
+bool dense_cluster_runs(int n) {
+  return n <= kCoarseDenseMax && dense_cluster_runs(kInvCtas, kInvThreads, inv_smem_bytes(n));
+}
+void dense_invert(int n, double *a, double *inv, int *status, cudaStream_t s, bool cluster, const int *unit) {
+  if (cluster) {
     launch_cluster(k_dense_invert_cluster, kInvCtas, 1, kInvThreads, inv_smem_bytes(n), s, n, (const double *)a, inv,
                    status, unit);
     CHNSS_LAUNCH_CK();

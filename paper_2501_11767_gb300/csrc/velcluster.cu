@@ -491,6 +491,15 @@ void transfer_tables(VlcDesc &d) {
     }
 }
 
+bool runs(bool bf16, bool open, int ctas, size_t smem) {
+  constexpr size_t most = kSmemLimit - sizeof(Fixed);
+  if (bf16)
+    return open ? cluster_runs<k_vel_cluster<__nv_bfloat16, true>>(ctas, kThreads, smem, most)
+                : cluster_runs<k_vel_cluster<__nv_bfloat16, false>>(ctas, kThreads, smem, most);
+  return open ? cluster_runs<k_vel_cluster<float, true>>(ctas, kThreads, smem, most)
+              : cluster_runs<k_vel_cluster<float, false>>(ctas, kThreads, smem, most);
+}
+
 }  // namespace
 
 VlcPlan vlc_plan(Arena &ar, const std::vector<const Level *> &lev, int open_top, const std::vector<P2Table> &tab,
@@ -504,7 +513,7 @@ VlcPlan vlc_plan(Arena &ar, const std::vector<const Level *> &lev, int open_top,
     if (first == (int)lev.size()) return plan;
     bool ok = layout(first, lev, open_top, degree, coarse_iter, d, plan.ctas, plan.smem);
     for (size_t l = first; ok && l + (coarse_iter ? 0 : 1) < lev.size(); ++l) ok = tab[l].ok;
-    if (ok) break;
+    if (ok && runs(val[first] == nullptr, open_top != 0, plan.ctas, plan.smem)) break;
   }
   transfer_tables(d);
   plan.bf16 = val[first] == nullptr;
@@ -534,7 +543,6 @@ template <typename VT, bool OPEN>
 void launch(const VlcPlan &p, cudaStream_t s) {
   Coef tab;
   for (int k = 0; k < 2 * (kP2Slots + kP2TopSlots); ++k) tab.c[k] = p.tab[k];
-  allow_cluster<k_vel_cluster<VT, OPEN>>(kSmemLimit - sizeof(Fixed));
   launch_cluster(k_vel_cluster<VT, OPEN>, p.ctas, 1, kThreads, p.smem, s, (const VlcDesc *)p.desc, tab);
   CHNSS_LAUNCH_CK();
 }

@@ -59,7 +59,8 @@ struct VlcPlan {
 };
 
 // Plan for the coarse end of an FP32 hierarchy (values FP32, or BF16 in val16)
-// whose levels are in stencil order; first = -1 if no level fits.
+// whose levels are in stencil order; first = -1 if no level fits or the
+// device has no place for its cluster.
 VlcPlan vlc_plan(Arena &ar, const std::vector<const Level *> &lev, int open_top, const std::vector<P2Table> &tab,
                  const std::vector<float *> &val, const std::vector<__nv_bfloat16 *> &val16,
                  const std::vector<float *> &dinv, const std::vector<double *> &coef, const std::vector<float *> &b,
