@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(mgc_threads<T>()) k_p1_cluster(const MgcDesc<T
       const double *row = d.cinv + (long)r * d.nc;
       double s = 0.0;
 #pragma unroll 8
-      for (int c = 0; c < d.nc; ++c) s += row[c] * (double)b[c];
+      for (int c = 0; c < d.nc; ++c) s = fma(row[c], (double)b[c], s);
       for (int z = 0; z < ctas; ++z) *cl.map_shared_rank(sm + q.x_off + k * q.vec + at + r, z) = (T)s;
     }
   } else if (me == 0 && d.na < d.nlev) {   // one-block levels
@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(mgc_threads<T>()) k_p1_cluster(const MgcDesc<T
           const double *row = d.cinv + (long)r * d.nc;
           double s = 0.0;
 #pragma unroll 8
-          for (int c = 0; c < d.nc; ++c) s += row[c] * (double)b[c];
+          for (int c = 0; c < d.nc; ++c) s = fma(row[c], (double)b[c], s);
           sm[q.x_off + k * q.vec + 1 + q.w + r] = (T)s;
         }
         __syncthreads();

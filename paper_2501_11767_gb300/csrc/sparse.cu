@@ -31,10 +31,7 @@ __device__ __forceinline__ T group_sum(T v) {
 // Chebyshev step of one row: c0 u + c2 dinv (b - A u) (+ c1 w)
 template <typename T>
 __device__ __forceinline__ T cheb_row(const double *coef, T ui, T di, T bi, T acc, bool has_w, T wi) {
-  const T c0 = (T)coef[0], c1 = (T)coef[1], c2 = (T)coef[2];
-  T v = c0 * ui + c2 * di * (bi - acc);
-  if (has_w) v += c1 * wi;
-  return v;
+  return cheb_step<T>((T)coef[0], (T)coef[1], (T)coef[2], ui, di, bi, acc, has_w, wi);
 }
 
 template <typename T>
@@ -208,9 +205,6 @@ __device__ __forceinline__ void load_blk(const double *p, double b[4]) {
   b[0] = v0.x; b[1] = v0.y; b[2] = v1.x; b[3] = v1.y;
 }
 
-__device__ __forceinline__ double fma_t(double a, double b, double c) { return fma(a, b, c); }
-__device__ __forceinline__ float fma_t(float a, float b, float c) { return fmaf(a, b, c); }
-
 template <typename T> __device__ __forceinline__ T from_double(double x) { return (T)x; }
 template <> __device__ __forceinline__ __nv_bfloat16 from_double<__nv_bfloat16>(double x) {
   return __double2bfloat16(x);   // round to nearest even
@@ -298,7 +292,7 @@ __global__ void __launch_bounds__(K >= 8 ? 32 * K : 256) k_sell_split(int nslice
     const int *cp = col + b0 + lane;
     const VT *vp = val + b0 + lane;
 #pragma unroll 4
-    for (int j = k; j < w; j += K) acc += ldv(vp + j * 32) * u[cp[j * 32]];
+    for (int j = k; j < w; j += K) acc = fma_of((T)ldv(vp + j * 32), u[cp[j * 32]], acc);
   }
   part[ls][k][lane] = acc;
   __syncthreads();
@@ -340,8 +334,8 @@ __global__ void __launch_bounds__(256) k_sell_bsr2_split(int nslices, const int 
       T b[4];
       load_blk(val + 4 * e, b);
       const T x0 = u[2L * c], x1 = u[2L * c + 1];
-      acc0 = fma_t(b[1], x1, fma_t(b[0], x0, acc0));
-      acc1 = fma_t(b[3], x1, fma_t(b[2], x0, acc1));
+      acc0 = fma_of(b[1], x1, fma_of(b[0], x0, acc0));
+      acc1 = fma_of(b[3], x1, fma_of(b[2], x0, acc1));
     }
   }
   part[ls][k][0][lane] = acc0;
@@ -377,9 +371,9 @@ __global__ void __launch_bounds__(K >= 8 ? 32 * K : 256) k_sell_bsr3(int nslices
   auto fma_blk = [&](const T (&v)[9], const T (&x)[3]) {
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
-      acc[r] = fma_t(v[3 * r], x[0], acc[r]);
-      acc[r] = fma_t(v[3 * r + 1], x[1], acc[r]);
-      acc[r] = fma_t(v[3 * r + 2], x[2], acc[r]);
+      acc[r] = fma_of(v[3 * r], x[0], acc[r]);
+      acc[r] = fma_of(v[3 * r + 1], x[1], acc[r]);
+      acc[r] = fma_of(v[3 * r + 2], x[2], acc[r]);
     }
   };
   if (slice < nslices) {
@@ -464,9 +458,9 @@ __global__ void __launch_bounds__(1024) k_cheb_bsr3_block(int nslices, int K, co
         const T x0 = cur[3 * c], x1 = cur[3 * c + 1], x2 = cur[3 * c + 2];
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
-          acc[r] = fma_t(ldv(vb + 32 * (3 * r)), x0, acc[r]);
-          acc[r] = fma_t(ldv(vb + 32 * (3 * r + 1)), x1, acc[r]);
-          acc[r] = fma_t(ldv(vb + 32 * (3 * r + 2)), x2, acc[r]);
+          acc[r] = fma_of(ldv(vb + 32 * (3 * r)), x0, acc[r]);
+          acc[r] = fma_of(ldv(vb + 32 * (3 * r + 1)), x1, acc[r]);
+          acc[r] = fma_of(ldv(vb + 32 * (3 * r + 2)), x2, acc[r]);
         }
       }
     }
@@ -538,7 +532,7 @@ __global__ void __launch_bounds__(kSellMaxBlock) k_sell_w8(int nslices, const in
   T acc = 0;
 #pragma unroll
   for (int j = 0; j < 8; ++j)
-    if (j < w) acc += v[j] * u[c[j]];
+    if (j < w) acc = fma_of(v[j], u[c[j]], acc);
   if (row < 0) return;
   T r;
   if (mode == SPMV_PLAIN) r = acc;
@@ -582,7 +576,7 @@ __global__ void __launch_bounds__(kSellMaxBlock) k_stencil7(int nrows, StencilOf
   }
   T acc = 0;
 #pragma unroll
-  for (int j = 0; j < 7; ++j) acc += v[j] * u[c[j]];
+  for (int j = 0; j < 7; ++j) acc = fma_of(v[j], u[c[j]], acc);
   T r;
   if (mode == SPMV_PLAIN) r = acc;
   else if (mode == SPMV_RES) r = bi - acc;
@@ -619,8 +613,8 @@ __global__ void __launch_bounds__(kSellMaxBlock) k_sell_bsr2(int nslices, const 
     }
     // two FMAs per component (not a multiply, an FMA and an add): the FP64
     // form of this kernel is bound by the FP64 pipe
-    acc0 = fma_t(b[1], x1, fma_t(b[0], x0, acc0));
-    acc1 = fma_t(b[3], x1, fma_t(b[2], x0, acc1));
+    acc0 = fma_of(b[1], x1, fma_of(b[0], x0, acc0));
+    acc1 = fma_of(b[3], x1, fma_of(b[2], x0, acc1));
   }
   if (row < 0) return;
   epilogue<T>(mode, 2L * row, acc0, u, out, a, a.coef);
@@ -1396,7 +1390,7 @@ __global__ void k_dense_apply(int n, const double *inv, const T *b, T *x) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= n) return;
   double s = 0.0;
-  for (int c = 0; c < n; ++c) s += inv[(long)r * n + c] * (double)b[c];
+  for (int c = 0; c < n; ++c) s = fma(inv[(long)r * n + c], (double)b[c], s);
   x[r] = (T)s;
 }
 
@@ -1450,7 +1444,7 @@ __device__ __forceinline__ void sell_w8m_slice(int slice, int lane, const int *s
     for (int k = 0; k < NR; ++k)
 #pragma unroll
       for (int j = 0; j < 8; ++j)
-        if (j0 + j < w) acc[k] += v[j] * u.p[k][c[j]];
+        if (j0 + j < w) acc[k] = fma_of(v[j], u.p[k][c[j]], acc[k]);
   }
   if (row < 0) return;
 #pragma unroll
@@ -1499,7 +1493,7 @@ __global__ void __launch_bounds__(kSellMaxBlock) k_stencil7m(int nrows, StencilO
   for (int k = 0; k < NR; ++k) {
     acc[k] = 0;
 #pragma unroll
-    for (int j = 0; j < 7; ++j) acc[k] += v[j] * u.p[k][c[j]];
+    for (int j = 0; j < 7; ++j) acc[k] = fma_of(v[j], u.p[k][c[j]], acc[k]);
   }
 #pragma unroll
   for (int k = 0; k < NR; ++k) {
@@ -1594,7 +1588,7 @@ __global__ void __launch_bounds__(512) k_mg_tail(const TailDesc<T> *__restrict__
     for (int r = threadIdx.x; r < d.nc; r += blockDim.x)
       for (int k = 0; k < NR; ++k) {
         double s = 0.0;
-        for (int c = 0; c < d.nc; ++c) s += d.cinv[(long)r * d.nc + c] * (double)q.b.p[k][c];
+        for (int c = 0; c < d.nc; ++c) s = fma(d.cinv[(long)r * d.nc + c], (double)q.b.p[k][c], s);
         q.x.p[k][r] = (T)s;
       }
     __syncthreads();
@@ -1639,7 +1633,7 @@ __global__ void k_dense_apply_m(int n, int nr, const double *inv, MultiPtr<T> b,
   if (r >= n) return;
   for (int k = 0; k < nr; ++k) {
     double s = 0.0;
-    for (int c = 0; c < n; ++c) s += inv[(long)r * n + c] * (double)b.p[k][c];
+    for (int c = 0; c < n; ++c) s = fma(inv[(long)r * n + c], (double)b.p[k][c], s);
     x.p[k][r] = (T)s;
   }
 }
