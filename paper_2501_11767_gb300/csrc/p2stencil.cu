@@ -1,4 +1,8 @@
 // P2 velocity stencil kernels (see p2stencil.h).
+#include <math_constants.h>
+
+#include <cmath>
+
 #include "p2slots.h"
 
 namespace chnss {
@@ -231,7 +235,7 @@ __global__ void k_p2_table(int n, int open, const int *__restrict__ rowptr, cons
   if (k >= kP2Slots + kP2TopSlots) return;
   const int m = 2 * n + 1, s = k < kP2Slots ? k : k - kP2Slots;
   const int ty = s < 19 ? 0 : (s - 10) / 9;
-  c[2 * k] = c[2 * k + 1] = 0.0;
+  c[2 * k] = c[2 * k + 1] = CUDART_NAN;   // no such coupling
   const int I = 2 * (n / 2) + (ty & 1), J = k < kP2Slots ? 2 * (n / 2) + (ty >> 1) : 2 * n;
   if (prescribed(I, J, m, open) || J + c_slots.dj[s] >= m) return;
   // a coupling to a prescribed node holds zeros: take it from another row of the type
@@ -298,6 +302,10 @@ P2Table p2_table(Arena &keep, const Level &L, int open_top, const double *A, cud
   CHNSS_CK(cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
   CHNSS_CK(cudaStreamSynchronize(s));
   t.ok = hbad == 0;
+  for (int k = 0; k < kP2Slots + kP2TopSlots; ++k) {
+    t.seen[k] = !std::isnan(t.c[2 * k]);
+    if (!t.seen[k]) t.c[2 * k] = t.c[2 * k + 1] = 0.0;
+  }
   std::vector<float> f(t.c, t.c + kCount), h(kCount);
   for (int k = 0; k < kCount; ++k) h[k] = __bfloat162float(__double2bfloat16(t.c[k]));
   t.d32 = keep.upload(f);

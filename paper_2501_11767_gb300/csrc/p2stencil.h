@@ -27,6 +27,13 @@ struct P2Table {
   // device copies: rounded to FP32, rounded to BF16 (as FP32)
   const float *d32 = nullptr, *d16 = nullptr;
   bool ok = false;                               // every row of the level matches it
+  bool seen[kP2Slots + kP2TopSlots] = {};        // the level couples two free nodes by the slot (else: zeros)
+  // o's entries hold for this level as well: equal wherever it has the coupling
+  bool holds(const P2Table &o) const {
+    for (int k = 0; k < kP2Slots + kP2TopSlots; ++k)
+      if (seen[k] && !(o.seen[k] && o.c[2 * k] == c[2 * k] && o.c[2 * k + 1] == c[2 * k + 1])) return false;
+    return true;
+  }
 };
 
 inline long p2_ld(int n) { return ((long)(n + 1) * (n + 1) + 31) / 32 * 32; }

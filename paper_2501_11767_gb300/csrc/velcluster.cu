@@ -512,7 +512,8 @@ VlcPlan vlc_plan(Arena &ar, const std::vector<const Level *> &lev, int open_top,
   for (;; ++first) {
     if (first == (int)lev.size()) return plan;
     bool ok = layout(first, lev, open_top, degree, coarse_iter, d, plan.ctas, plan.smem);
-    for (size_t l = first; ok && l + (coarse_iter ? 0 : 1) < lev.size(); ++l) ok = tab[l].ok;
+    // one table for all of them
+    for (size_t l = first; ok && l + (coarse_iter ? 0 : 1) < lev.size(); ++l) ok = tab[l].ok && tab[l].holds(tab[first]);
     if (ok && runs(val[first] == nullptr, open_top != 0, plan.ctas, plan.smem)) break;
   }
   transfer_tables(d);
