@@ -324,6 +324,27 @@ chnss_status chnss_debug_cluster_runs(int ctas, int threads, long smem, int *run
  * none), levels swept as a P2 stencil.  Allocates and synchronises. */
 chnss_status chnss_debug_vcycle(chnss_ctx_t ctx, int block, int precision, int clusters, int nvec, const double *in,
                                 double *out, int *info);
+/* Test entry: one sweep of the assembled velocity block of a level (0: the
+ * finest) with FP32 vectors.  layout 0: 2x2-block SELL; 1: P2 stencil
+ * (CHNSS_ERR_STATE if the level is not one).  precision 1: FP32 values; 2:
+ * BF16.  mode as chnss_debug_spmv; coef[4]: the scale of a first iterate,
+ * then (c0, c1, c2).  start (mode 3, stencil): 0: iterates from u and w (may
+ * be null); 1: u = coef[0] dinv b, formed in the sweep; 2: u from u, w =
+ * coef[0] dinv b.  HOST arrays of 2 N2 values of the level; out is read by
+ * mode 2.  *warps (optional): warps a slice or row. */
+chnss_status chnss_debug_velocity_sweep(chnss_ctx_t ctx, int level, int layout, int precision, int mode, int start,
+                                        const double *u, const double *b, const double *w, const double *dinv,
+                                        const double *coef, double *out, int *warps);
+/* Test entry: a grid transfer of the velocity between level and level + 1,
+ * precision 0 (FP64) or 1 (FP32).  up 0: out (coarse) = R in (fine); 1: out
+ * (fine) += P in (coarse).  HOST arrays. */
+chnss_status chnss_debug_velocity_transfer(chnss_ctx_t ctx, int level, int precision, int up, const double *in,
+                                           double *out);
+/* Test entry: the dense inverse of a coarsest level, by a cluster (n <= 256)
+ * or by one block.  unit (may be null, n even): n / 2 flags, nonzero where
+ * rows and columns 2 i, 2 i + 1 are the identity's.  HOST arrays; *status 1
+ * if a pivot was exactly zero. */
+chnss_status chnss_debug_dense_inverse(int n, const double *a, const int *unit, int cluster, double *inv, int *status);
 /* Assembled right-hand side of a system (host, chnss_system_size doubles). */
 chnss_status chnss_export_rhs(chnss_ctx_t ctx, chnss_system sys, double *host_out);
 

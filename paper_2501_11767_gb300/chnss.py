@@ -143,6 +143,11 @@ EXPORTS = {
     "chnss_debug_cluster_runs": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_long,
                                                 ctypes.POINTER(ctypes.c_int)]),
     "chnss_debug_vcycle": (ctypes.c_int, [ctypes.c_void_p] + [ctypes.c_int] * 4 + [ctypes.c_void_p] * 3),
+    "chnss_debug_velocity_sweep": (ctypes.c_int, [ctypes.c_void_p] + [ctypes.c_int] * 5 + [ctypes.c_void_p] * 6 +
+                                   [ctypes.POINTER(ctypes.c_int)]),
+    "chnss_debug_velocity_transfer": (ctypes.c_int, [ctypes.c_void_p] + [ctypes.c_int] * 3 + [ctypes.c_void_p] * 2),
+    "chnss_debug_dense_inverse": (ctypes.c_int, [ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int,
+                                                 ctypes.c_void_p, ctypes.POINTER(ctypes.c_int)]),
     "chnss_profile_enable": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int]),
     "chnss_profile_read": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(Profile)]),
     "chnss_inner_stats_read": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.POINTER(InnerStats)]),
@@ -481,6 +486,29 @@ class Context:
                                          out.ctypes.data, info.ctypes.data), self._h)
         return (out, *info.tolist())
 
+    def debug_velocity_sweep(self, level: int, layout: int, precision: int, mode: int, u, b=None, w=None, dinv=None,
+                             coef=None, out=None, start: int = 0):
+        """chnss_debug_velocity_sweep: (result, warps a slice or row)."""
+        size = 2 * (2 * (self.mesh.n >> level) + 1) ** 2
+        arr = lambda a, k: None if a is None else np.ascontiguousarray(a, dtype=np.float64).reshape(k)   # noqa: E731
+        u, b, w, dinv, coef = arr(u, size), arr(b, size), arr(w, size), arr(dinv, size), arr(coef, 4)
+        out = np.zeros(size) if out is None else np.array(out, dtype=np.float64).reshape(size)
+        ptr = lambda a: None if a is None else a.ctypes.data   # noqa: E731
+        k = ctypes.c_int()
+        _check(load().chnss_debug_velocity_sweep(self._h, level, layout, precision, mode, start, ptr(u), ptr(b),
+                                                 ptr(w), ptr(dinv), ptr(coef), out.ctypes.data, ctypes.byref(k)),
+               self._h)
+        return out, k.value
+
+    def debug_velocity_transfer(self, level: int, precision: int, up: bool, x, out=None):
+        """chnss_debug_velocity_transfer: R x, or out + P x."""
+        nf, ng = (2 * (2 * (self.mesh.n >> k) + 1) ** 2 for k in (level, level + 1))
+        x = np.ascontiguousarray(x, dtype=np.float64).reshape(ng if up else nf)
+        out = np.zeros(nf if up else ng) if out is None else np.array(out, dtype=np.float64).reshape(nf)
+        _check(load().chnss_debug_velocity_transfer(self._h, level, precision, 1 if up else 0, x.ctypes.data,
+                                                    out.ctypes.data), self._h)
+        return out
+
     def export_rhs(self, sys: int):
         out = np.zeros(self.system_size(sys), dtype=np.float64)
         _check(load().chnss_export_rhs(self._h, sys, out.ctypes.data), self._h)
@@ -623,6 +651,16 @@ def debug_cluster_runs(ctas: int, threads: int, smem: int) -> bool:
     out = ctypes.c_int()
     _check(load().chnss_debug_cluster_runs(ctas, threads, smem, ctypes.byref(out)))
     return out.value != 0
+
+
+def debug_dense_inverse(a, cluster: bool, unit=None):
+    """chnss_debug_dense_inverse: (inverse, status)."""
+    a = np.ascontiguousarray(a, dtype=np.float64)
+    inv, st = np.zeros_like(a), ctypes.c_int()
+    unit = None if unit is None else np.ascontiguousarray(unit, dtype=np.int32)
+    _check(load().chnss_debug_dense_inverse(len(a), a.ctypes.data, None if unit is None else unit.ctypes.data,
+                                            1 if cluster else 0, inv.ctypes.data, ctypes.byref(st)))
+    return inv, st.value
 
 
 def debug_cgs2(V, w, arith: int):

@@ -1566,6 +1566,67 @@ void run(chnss_ctx *c, int block, bool bf16, bool clusters, int nvec, const doub
   for (int l = 0; l < h.nl; ++l) info[3] += h.stencil(l) ? 1 : 0;
 }
 
+// n host values as T on the device, and back
+template <typename T>
+T *upload(ScopedDeviceMem &mem, const double *h, long n) {
+  std::vector<T> v(n);
+  for (long i = 0; i < n; ++i) v[i] = (T)h[i];
+  T *d = mem.get<T>(n);
+  CHNSS_CK(cudaMemcpy(d, v.data(), n * sizeof(T), cudaMemcpyHostToDevice));
+  return d;
+}
+template <typename T>
+void download(const T *d, long n, double *h, cudaStream_t s) {
+  std::vector<T> v(n);
+  CHNSS_CK(cudaMemcpyAsync(v.data(), d, n * sizeof(T), cudaMemcpyDeviceToHost, s));
+  CHNSS_CK(cudaStreamSynchronize(s));
+  for (long i = 0; i < n; ++i) h[i] = (double)v[i];
+}
+
+// One sweep of chnss_debug_velocity_sweep with values VT.
+template <typename VT>
+void sweep(chnss_ctx *c, int level, bool stencil, int mode, int start, const double *u, const double *b,
+           const double *w, const double *dinv, const double *coef, double *out) {
+  const Level &L = c->lv(level);
+  const long n = 2L * L.N2, nv = stencil ? p2_values_count(L.n) : 4L * L.p2.sell.nent;
+  const int open = c->mesh->m.top_bc;
+  cudaStream_t s = c->s;
+  CHNSS_CK(cudaStreamSynchronize(s));
+  ScopedDeviceMem mem;
+  VT *val = mem.get<VT>(nv);
+  const float *du = upload<float>(mem, u, n);
+  float *dout = upload<float>(mem, out, n);
+  SpmvArgs a;
+  if (b) a.b = upload<float>(mem, b, n);
+  if (w) a.w = upload<float>(mem, w, n);
+  if (dinv) a.dinv = upload<float>(mem, dinv, n);
+  const double *dc = coef ? upload<double>(mem, coef, 4) : nullptr;
+  if (coef) a.coef = dc + 1;
+  if (stencil) {
+    p2_values<VT>(L, open, c->A[level], val, s);
+    p2_spmv<VT>(L, open, c->p2tab[level], val, du, dout, (SpmvMode)mode, a, (P2Start)start, dc, s);
+  } else {
+    sell_gather<VT>(L.p2.sell, 4, c->A[level], val, s);
+    if constexpr (std::is_same<VT, float>::value) spmv_sell_bsr2<float>(L.p2, val, du, dout, (SpmvMode)mode, a, s);
+    else spmv_sell_bsr2(L.p2, val, du, dout, (SpmvMode)mode, a, s);
+  }
+  download(dout, n, out, s);
+}
+
+template <typename T>
+void transfer(chnss_ctx *c, int level, bool up, const double *in, double *out) {
+  const Level &F = c->lv(level), &G = c->lv(level + 1);
+  const long nf = 2L * F.N2, ng = 2L * G.N2;
+  cudaStream_t s = c->s;
+  CHNSS_CK(cudaStreamSynchronize(s));
+  ScopedDeviceMem mem;
+  const T *di = upload<T>(mem, in, up ? ng : nf);
+  T *dout = upload<T>(mem, out, up ? nf : ng);
+  if (up) p2_prolong_add<T>(G.n, c->mesh->m.top_bc, di, dout, s);
+  else p2_restrict<T>(G.n, c->mesh->m.top_bc, di, dout, s);
+  download(dout, up ? nf : ng, out, s);
+}
+
 }  // namespace debug_vcycle_detail
 }  // namespace chnss
 
@@ -1862,6 +1923,62 @@ chnss_status chnss_debug_vcycle(chnss_ctx_t ctx, int block, int precision, int c
   else debug_vcycle_detail::run<float>(ctx, block, precision == 2, clusters != 0, nvec, in, out, info);
   return CHNSS_OK;
   ABI_CATCH(ctx)
+}
+
+chnss_status chnss_debug_velocity_sweep(chnss_ctx_t ctx, int level, int layout, int precision, int mode, int start,
+                                        const double *u, const double *b, const double *w, const double *dinv,
+                                        const double *coef, double *out, int *warps) {
+  if (!ctx) return fail(nullptr, CHNSS_ERR_ARG, "null context");
+  ABI_TRY
+  if (level < 0 || level >= ctx->nlev) throw Error{CHNSS_ERR_ARG, "level out of range"};
+  if (layout != 0 && layout != 1) throw Error{CHNSS_ERR_ARG, "layout must be 0 (2x2-block SELL) or 1 (stencil)"};
+  if (precision != 1 && precision != 2) throw Error{CHNSS_ERR_ARG, "precision must be 1 or 2"};
+  if (mode < 0 || mode > 3 || start < 0 || start > 2) throw Error{CHNSS_ERR_ARG, "mode must be 0..3 and start 0..2"};
+  if (start != 0 && (mode != SPMV_CHEB || layout != 1 || w))
+    throw Error{CHNSS_ERR_ARG, "starts 1 and 2: Chebyshev sweeps of the stencil, without w"};
+  if (!u || !out || ((mode == 1 || mode == 3) && !b) || (mode == 3 && (!dinv || !coef)))
+    throw Error{CHNSS_ERR_ARG, "null argument"};
+  if (!ctx->assembled) throw Error{CHNSS_ERR_STATE, "a sweep needs an assembled context"};
+  if (layout == 1 && !p2_applies(ctx->lv(level), ctx->p2tab[level], 4)) throw Error{CHNSS_ERR_STATE, "the level is not a P2 stencil"};
+  if (precision == 1) debug_vcycle_detail::sweep<float>(ctx, level, layout == 1, mode, start, u, b, w, dinv, coef, out);
+  else debug_vcycle_detail::sweep<__nv_bfloat16>(ctx, level, layout == 1, mode, start, u, b, w, dinv, coef, out);
+  if (warps) *warps = sell_warps_bsr2(ctx->lv(level).p2.sell);
+  return CHNSS_OK;
+  ABI_CATCH(ctx)
+}
+
+chnss_status chnss_debug_velocity_transfer(chnss_ctx_t ctx, int level, int precision, int up, const double *in,
+                                           double *out) {
+  if (!ctx) return fail(nullptr, CHNSS_ERR_ARG, "null context");
+  ABI_TRY
+  if (level < 0 || level + 1 >= ctx->nlev) throw Error{CHNSS_ERR_ARG, "level out of range"};
+  if (precision != 0 && precision != 1) throw Error{CHNSS_ERR_ARG, "precision must be 0 or 1"};
+  if (!in || !out) throw Error{CHNSS_ERR_ARG, "null argument"};
+  if (precision == 0) debug_vcycle_detail::transfer<double>(ctx, level, up != 0, in, out);
+  else debug_vcycle_detail::transfer<float>(ctx, level, up != 0, in, out);
+  return CHNSS_OK;
+  ABI_CATCH(ctx)
+}
+
+chnss_status chnss_debug_dense_inverse(int n, const double *a, const int *unit, int cluster, double *inv, int *status) {
+  ABI_TRY
+  if (n < 1 || !a || !inv || !status) throw Error{CHNSS_ERR_ARG, "bad size or null argument"};
+  if (unit && n % 2 != 0) throw Error{CHNSS_ERR_ARG, "unit pairs need an even size"};
+  if (cluster && !dense_cluster_runs(n)) throw Error{CHNSS_ERR_ARG, "no cluster for this size"};
+  const long nn = (long)n * n;
+  ScopedDeviceMem mem;
+  cudaStream_t s = nullptr;
+  double *da = debug_vcycle_detail::upload<double>(mem, a, nn), *di = mem.get<double>(nn);
+  int *ds = mem.get<int>(1), *du = nullptr;
+  if (unit) {
+    du = mem.get<int>(n / 2);
+    CHNSS_CK(cudaMemcpy(du, unit, n / 2 * sizeof(int), cudaMemcpyHostToDevice));
+  }
+  dense_invert(n, da, di, ds, s, cluster != 0, du);
+  debug_vcycle_detail::download(di, nn, inv, s);
+  CHNSS_CK(cudaMemcpy(status, ds, sizeof(int), cudaMemcpyDeviceToHost));
+  return CHNSS_OK;
+  ABI_CATCH(nullptr)
 }
 
 chnss_status chnss_debug_spmv(int layout, int precision, int mode, int nrows, int ncols, const int *rowptr,
