@@ -3,16 +3,19 @@ of the exported blocks and, bit for bit, against the 2x2-block SELL sweep
 (the same sums in the same order) on every level, in its four epilogues and
 three starts, FP32 and BF16 values, both top conditions and a non-square box,
 at sizes that reach one cell a thread (256) and 2, 4 and 8 warps a row (176,
-128, 6); the dense inverse of a coarsest level by a cluster and by one block."""
+128, 6); the grid transfers against the oracle's; the dense inverse of a
+coarsest level by a cluster and by one block."""
 import numpy as np
 import pytest
 import scipy.sparse as sp
 
+from oracle import mg
+from oracle.mesh import Mesh
 from paper_2501_11767_gb300 import chnss, inputs
 
 pytestmark = pytest.mark.gpu
 
-EPS = 2.0 ** -24
+EPS = {0: 2.0 ** -53, 1: 2.0 ** -24}
 COEF = [0.37, 1.21, -0.43, 0.77]                    # scale, c0, c1, c2
 
 
@@ -49,6 +52,7 @@ FORMS = [(0, 0, False), (1, 0, False), (2, 0, False), (3, 0, False), (3, 0, True
 def test_sweep(n, lxy, warps, top_bc):
     ctx = _context(n, top_bc, lxy)
     rp, col, val = ctx.export_csr(chnss.MAT_A)
+    eps = EPS[1]
     c = np.asarray(COEF, dtype=np.float32).astype(np.float64)
     for level in range(ctx.mesh.levels):
         size = 2 * (2 * (n >> level) + 1) ** 2
@@ -84,7 +88,26 @@ def test_sweep(n, lxy, warps, top_bc):
                     if ww is not None:
                         want, scale = want + c[2] * ww, scale + np.abs(c[2] * ww)
                 # sums of at most 38 products and six more roundings
-                assert (np.abs(got - want) <= 48 * EPS * scale).all(), where
+                assert (np.abs(got - want) <= 48 * eps * scale).all(), where
+
+
+@pytest.mark.parametrize("top_bc", [0, 1])
+@pytest.mark.parametrize("n", [4, 6, 10, 44, 200])         # 200: lines of more than one block of threads
+def test_transfers(n, top_bc):
+    ctx = _context(n, top_bc, (1.0, 1.0))
+    fine, coarse = (Mesh(k, top_free=top_bc == 1) for k in (n, n // 2))
+    P = mg.prolongation_velocity(coarse, fine)
+    rng = np.random.default_rng(n)
+    for precision in (0, 1):
+        t = np.float32 if precision else np.float64
+        r, x = (rng.standard_normal(k).astype(t).astype(np.float64) for k in P.shape)
+        got = ctx.debug_velocity_transfer(0, precision, False, r)
+        want = P.T @ r
+        # at most 25 terms with exact weights
+        assert (np.abs(got - want) <= 26 * EPS[precision] * (abs(P.T) @ np.abs(r))).all(), precision
+        got = ctx.debug_velocity_transfer(0, precision, True, x, out=r)
+        want = r + P @ x
+        assert (np.abs(got - want) <= 8 * EPS[precision] * (np.abs(r) + abs(P) @ np.abs(x))).all(), precision
 
 
 @pytest.mark.parametrize("n", [1, 2, 50, 97, 98, 127, 128, 129, 224, 225, 242, 256])
