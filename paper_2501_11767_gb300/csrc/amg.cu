@@ -767,6 +767,7 @@ struct AmgHandle {
     }
     CHNSS_CK(cudaStreamEndCapture(s, &graph));
     g.kernels = g_launch_count.load() - before;
+    g_launch_count.fetch_sub(g.kernels, std::memory_order_relaxed);   // recorded, not launched
     const cudaError_t e = cudaGraphInstantiate(&g.exec, graph, 0);
     cudaGraphDestroy(graph);
     CHNSS_CK(e);
