@@ -355,7 +355,8 @@ chnss_status chnss_export_rhs(chnss_ctx_t ctx, chnss_system sys, double *host_ou
  * SpMV, Krylov orthogonalisation (one record per Arnoldi step), assembly
  * with preconditioner setup (bytes not counted), and the time of every
  * multigrid level below the finest, per V-cycle, for the P1 and the velocity
- * hierarchies (bytes not counted). */
+ * hierarchies (bytes not counted; of every level, where one launch takes the
+ * whole cycle: the fine-level families have no launches then). */
 typedef struct {
   long long launches;          /* kernels launched by the library in this process */
   int nkinds;

@@ -107,18 +107,19 @@ void Profiler::release() {
 namespace {
 // algorithmic bytes of one SpMV launch: values + column indices + row
 // pointers + one read of u, one write of out, plus the extra vector streams
-// of the epilogue (b for RES, b + dinv (+ w) for CHEB, out read for ADD)
+// of the epilogue (b for RES, b + dinv (+ w) for CHEB, out read for ADD); a
+// Chebyshev sweep that forms its first iterate reads no u (has_u false)
 // Algorithmic bytes of one sweep: every stored nonzero once (value, plus a
 // 4-byte column and the row pointers unless the stencil layout implies
 // them), the input and output vectors once, and the epilogue's vectors.
 double spmv_bytes(long nrows, long nnz, int vals_per_entry, long vec_len, size_t sv, size_t s, SpmvMode mode,
-                  bool has_w, bool implicit_index) {
+                  bool has_w, bool implicit_index, bool has_u = true) {
   double extra = 0.0;
   if (mode == SPMV_RES) extra = 1.0;
   if (mode == SPMV_ADD) extra = 1.0;
   if (mode == SPMV_CHEB) extra = has_w ? 3.0 : 2.0;
   const double index = implicit_index ? 0.0 : (double)nnz * 4.0 + 4.0 * (nrows + 1);
-  return (double)nnz * vals_per_entry * (double)sv + index + (2.0 + extra) * vec_len * s;
+  return (double)nnz * vals_per_entry * (double)sv + index + ((has_u ? 2.0 : 1.0) + extra) * vec_len * s;
 }
 }  // namespace
 
@@ -314,7 +315,7 @@ void MGHier<T>::op(int l, const T *u, T *out, SpmvMode mode, const SpmvArgs &a, 
                                       a.w != nullptr, false)
                          : spmv_bytes(pat[l]->nrows, pat[l]->nnz, kind == 0 ? 1 : stencil(l) ? 2 : 4, n[l],
                                       bf16 ? 2 : sizeof(T), sizeof(T), mode, a.w != nullptr && start == P2_PLAIN,
-                                      pat[l]->sell.stencil != 0 || stencil(l)));
+                                      pat[l]->sell.stencil != 0 || stencil(l), start != P2_FIRST));
 }
 
 template <typename T>
@@ -429,11 +430,15 @@ void MGHier<T>::vcycle(int l, cudaStream_t s) {
 template <typename T>
 void MGHier<T>::cycle(cudaStream_t s) {
   double *pb = ipartial ? ipartial : partial;
+  const int kc = kind == 0 ? Profiler::P1_MG_COARSE : Profiler::VEL_MG_COARSE;
+  const bool whole = prof && (mgc.first == 0 || vlc.first == 0);   // a cluster's whole cycle: timed as coarse levels
   if (singular) {
     vsum<T>(n[0], b[0], sum, pb, s);
     vec_sub_mean<T>((int)n[0], b[0], sum, s);
   }
+  const int tkc = whole ? prof->start(kc, s) : -1;
   vcycle(0, s);
+  if (whole) prof->stop(kc, tkc, s, 0.0);
   if (singular) {
     vsum<T>(n[0], x[0], sum, pb, s);
     vec_sub_mean<T>((int)n[0], x[0], sum, s);
@@ -714,7 +719,10 @@ void MGBatch<T>::vcycle(int l, cudaStream_t s) {
 
 template <typename T>
 void MGBatch<T>::apply(cudaStream_t s) {
+  Profiler *prof = mgc.first == 0 ? h->prof : nullptr;
+  const int tkc = prof ? prof->start(Profiler::P1_MG_COARSE, s) : -1;
   vcycle(0, s);
+  if (prof) prof->stop(Profiler::P1_MG_COARSE, tkc, s, 0.0);
 }
 
 template struct MGBatch<double>;
