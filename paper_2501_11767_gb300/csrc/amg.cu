@@ -875,7 +875,7 @@ struct AmgOperator : LinearOperator {
   long size() const override { return h->n; }
   void apply(const double *x, double *y, cudaStream_t s) override {
     SpmvArgs none;
-    spmv_sell<double>(h->lv[0]->A, h->a0sell, 1, x, y, SPMV_PLAIN, none, s);
+    spmv_sell<double>(h->lv[0]->A, h->a0sell, x, y, SPMV_PLAIN, none, s);
   }
   void precond(const double *r, double *z, cudaStream_t) override { h->vcycle(r, z); }
 };

@@ -283,7 +283,7 @@ void ch_precond(chnss_ctx *c, PrecSet<T> &P, int sp, double **slot, cudaStream_t
   vec_convert_from_slot<double, T>(N1, in, N1, X1.input(), s);
   X1.apply(s);
   SpmvArgs none;
-  spmv_sell<T>(c->lv(0).p1, P.Mv, 1, X1.output(), X2.input(), SPMV_PLAIN, none, s);
+  spmv_sell<T>(c->lv(0).p1, P.Mv, X1.output(), X2.input(), SPMV_PLAIN, none, s);
   X2.apply(s);
   X2.write_output(out, N1, s);
   join_side(c, s, 0);
@@ -348,7 +348,7 @@ void ns_precond(chnss_ctx *c, PrecSet<T> &P, double **slot, cudaStream_t s) {
   P.Kp.apply(q);
   SpmvArgs none;
   const Pattern &p1 = c->lv(0).p1;
-  spmv_sell<T>(p1, P.Apv, 1, P.Kp.output(), P.mb, SPMV_PLAIN, none, q);
+  spmv_sell<T>(p1, P.Apv, P.Kp.output(), P.mb, SPMV_PLAIN, none, q);
   // M_p^-1 by Chebyshev iteration of degree 5 on D^-1 M, spectrum [1/2, 2]
   vec_scale_dinv<T>(N1, c->massc, P.mdinv, P.mb, P.mx, q);
   SpmvArgs a;
@@ -358,7 +358,7 @@ void ns_precond(chnss_ctx *c, PrecSet<T> &P, double **slot, cudaStream_t s) {
   for (int k = 1; k <= 4; ++k) {
     a.coef = c->massc + 1 + 3 * (k - 1);
     a.w = k == 1 ? nullptr : other;
-    spmv_sell<T>(p1, P.Mv, 1, cur, other, SPMV_CHEB, a, q);
+    spmv_sell<T>(p1, P.Mv, cur, other, SPMV_CHEB, a, q);
     std::swap(cur, other);
   }
   vec_convert_to_slot<T, double>(N1, cur, out, nv, q);
@@ -488,18 +488,11 @@ struct ACOp : LinearOperator {
   long size() const override { return c->N1; }
   void apply(const double *x, double *y, cudaStream_t s) override {
     SpmvArgs none;
-    spmv_sell<double>(c->lv(0).p1, c->ACs, 1, x, y, SPMV_PLAIN, none, s);
+    spmv_sell<double>(c->lv(0).p1, c->ACs, x, y, SPMV_PLAIN, none, s);
   }
   void precond(const double *r, double *z, cudaStream_t s) override { run_prec(c, 3, r, z, s); }
   void after_sync() override { harvest_probes(c, 3); }
 };
-
-// y = A x on the fine velocity block (2x2-block SELL values)
-void apply_velocity(chnss_ctx *c, const double *val, const double *x, double *y, cudaStream_t s) {
-  const Level &F = c->lv(0);
-  SpmvArgs none;
-  spmv_sell_bsr2<double>(F.p2, val, x, y, SPMV_PLAIN, none, s);
-}
 
 struct NSOp : LinearOperator {
   chnss_ctx *c;
@@ -507,11 +500,11 @@ struct NSOp : LinearOperator {
   long size() const override { return 2L * c->N2 + c->N1; }
   void apply(const double *x, double *y, cudaStream_t s) override {
     const long nv = 2L * c->N2;
+    SpmvArgs none;
     const Pattern &p2 = c->lv(0).p2;
     const int tk = c->prof.start(Profiler::NS_OUTER_SPMV, s);
-    apply_velocity(c, c->As, x, y, s);
-    c->prof.stop(Profiler::NS_OUTER_SPMV, tk, s,
-                 (double)p2.nnz * 36.0 + 4.0 * (p2.nrows + 1) + 2.0 * nv * 8.0);
+    spmv_sell_bsr2<double>(p2, c->As, x, y, SPMV_PLAIN, none, s);
+    c->prof.stop(Profiler::NS_OUTER_SPMV, tk, s, (double)p2.nnz * 36.0 + 4.0 * (p2.nrows + 1) + 2.0 * nv * 8.0);
     spmv_sell_bt_add(c->mesh->m.pbt, c->Bts, x + nv, y, s);
     spmv_sell_b(c->mesh->m.pb, c->Bs, x, y + nv, s);
   }
@@ -623,7 +616,6 @@ void init_precset(chnss_ctx *c, PrecSet<T> &P) {
     P.AC.init(ar, 0, false, p1s, d1s, vals(c->AC), t1s, c->partial_ch);
   }
   init_block(c, BLOCK_VELOCITY, ar, P.A);
-  c->As = ar.alloc<double>(4L * c->lv(0).p2.sell.nent);   // the fine operator applied inside FGMRES
   init_block(c, BLOCK_KP, ar, P.Kp);
   for (int sp = 0; sp < 3; ++sp) {
     std::vector<const double *> x1, x2;
@@ -779,6 +771,7 @@ void create_context(chnss_ctx *c) {
   c->ACs = ar.alloc<double>(nent1);
   c->Ks = ar.alloc<double>(nent1);
   c->Ms = ar.alloc<double>(nent1);
+  c->As = ar.alloc<double>(4L * F.p2.sell.nent);
   for (int l = 0; l < nl; ++l) c->p2tab.push_back(p2_table(ar, m.lv[l], m.top_bc, c->Aconst[l], s));
   sell_gather<double>(F.p1.sell, 1, c->K1[0], c->Ks, s);
   sell_gather<double>(F.p1.sell, 1, c->M1[0], c->Ms, s);
@@ -1516,11 +1509,11 @@ void debug_spmv_run(int layout, int mode, Pattern &P, const std::vector<int> &hm
     a.coef = dc;
   }
   if constexpr (std::is_same<VT, __nv_bfloat16>::value) {
-    if (layout == 0) spmv_sell(P, dval, 1, dx, dy, (SpmvMode)mode, a, s);
+    if (layout == 0) spmv_sell(P, dval, dx, dy, (SpmvMode)mode, a, s);
     else if (layout == 1) spmv_sell_bsr2(P, dval, dx, dy, (SpmvMode)mode, a, s);
     else spmv_sell_bsr3(P, dval, dx, dy, (SpmvMode)mode, a, s);
   } else {
-    if (layout == 0) spmv_sell<T>(P, dval, 1, dx, dy, (SpmvMode)mode, a, s);
+    if (layout == 0) spmv_sell<T>(P, dval, dx, dy, (SpmvMode)mode, a, s);
     else if (layout == 1) spmv_sell_bsr2<T>(P, dval, dx, dy, (SpmvMode)mode, a, s);
     else spmv_sell_bsr3<T>(P, dval, dx, dy, (SpmvMode)mode, a, s);
   }
@@ -1939,7 +1932,7 @@ chnss_status chnss_debug_velocity_sweep(chnss_ctx_t ctx, int level, int layout, 
   if (!u || !out || ((mode == 1 || mode == 3) && !b) || (mode == 3 && (!dinv || !coef)))
     throw Error{CHNSS_ERR_ARG, "null argument"};
   if (!ctx->assembled) throw Error{CHNSS_ERR_STATE, "a sweep needs an assembled context"};
-  if (layout == 1 && !p2_applies(ctx->lv(level), ctx->p2tab[level], 4)) throw Error{CHNSS_ERR_STATE, "the level is not a P2 stencil"};
+  if (layout == 1 && !p2_applies(ctx->p2tab[level], 4)) throw Error{CHNSS_ERR_STATE, "the level is not a P2 stencil"};
   if (precision == 1) debug_vcycle_detail::sweep<float>(ctx, level, layout == 1, mode, start, u, b, w, dinv, coef, out);
   else debug_vcycle_detail::sweep<__nv_bfloat16>(ctx, level, layout == 1, mode, start, u, b, w, dinv, coef, out);
   if (warps) *warps = sell_warps_bsr2(ctx->lv(level).p2.sell);
@@ -2129,7 +2122,7 @@ chnss_status mass_solve_noalloc(chnss_ctx *c, const double *b, double *x, chnss_
   KrylovWork view;                       // no storage of its own
   view.nmax = n;
   view.w = base;                         // r
-  view.V = base + n;                     // z, p, q
+  view.V = base + n;                     // two directions, q
   view.partial = base + 4L * kNoAllocMaxN1;
   view.sc = view.partial + kNoAllocPartials;
   view.counter = reinterpret_cast<int *>(view.sc + 8);
@@ -2204,7 +2197,7 @@ struct ACOpT : LinearOperator {
   long size() const override { return c->N1; }
   void apply(const double *x, double *y, cudaStream_t s) override {
     SpmvArgs none;
-    spmv_sell<double>(c->lv(0).p1, c->ACsT, 1, x, y, SPMV_PLAIN, none, s);
+    spmv_sell<double>(c->lv(0).p1, c->ACsT, x, y, SPMV_PLAIN, none, s);
   }
   void precond(const double *r, double *z, cudaStream_t s) override { run_prec(c, 3, r, z, s); }
   void after_sync() override { harvest_probes(c, 3); }
@@ -2216,7 +2209,8 @@ struct NSOpT : LinearOperator {   // [[A^T, B^T], [B, 0]]
   long size() const override { return 2L * c->N2 + c->N1; }
   void apply(const double *x, double *y, cudaStream_t s) override {
     const long nv = 2L * c->N2;
-    apply_velocity(c, c->AsT, x, y, s);
+    SpmvArgs none;
+    spmv_sell_bsr2<double>(c->lv(0).p2, c->AsT, x, y, SPMV_PLAIN, none, s);
     spmv_sell_bt_add(c->mesh->m.pbt, c->Bts, x + nv, y, s);
     spmv_sell_b(c->mesh->m.pb, c->Bs, x, y + nv, s);
   }

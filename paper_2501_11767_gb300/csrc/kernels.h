@@ -65,7 +65,7 @@ void sell_gather(const Sell &S, int ncomp, const double *csr_vals, Tout *out, cu
 // ncomp = 4 each 2x2 block is transposed as well)
 void sell_gather_transposed(const Sell &S, int ncomp, const double *csr_vals, double *out, cudaStream_t s);
 template <typename T>
-void spmv_sell(const Pattern &P, const T *sval, int ncomp, const T *u, T *out, SpmvMode mode, const SpmvArgs &a,
+void spmv_sell(const Pattern &P, const T *sval, const T *u, T *out, SpmvMode mode, const SpmvArgs &a,
                cudaStream_t s);
 template <typename T>
 void spmv_sell_bsr2(const Pattern &P, const T *sval, const T *u, T *out, SpmvMode mode, const SpmvArgs &a,
@@ -121,7 +121,7 @@ struct TailLevel {
   TailSell A, R, P;               // operator; restriction to / prolongation from the next level
   const T *val = nullptr, *Rval = nullptr, *Pval = nullptr, *dinv = nullptr;
   const double *coef = nullptr;   // Chebyshev coefficients of the level
-  MultiPtr<T> x, t, r, b;
+  T *x = nullptr, *t = nullptr, *r = nullptr, *b = nullptr;
 };
 template <typename T>
 struct TailDesc {
@@ -134,7 +134,7 @@ struct TailDesc {
 template <typename T>
 void mg_tail(const TailDesc<T> *d_desc, int width, cudaStream_t s);
 // BF16-stored values, FP32 vectors and accumulation (preconditioner variant)
-void spmv_sell(const Pattern &P, const __nv_bfloat16 *sval, int ncomp, const float *u, float *out, SpmvMode mode,
+void spmv_sell(const Pattern &P, const __nv_bfloat16 *sval, const float *u, float *out, SpmvMode mode,
                const SpmvArgs &a, cudaStream_t s);
 void spmv_sell_bsr2(const Pattern &P, const __nv_bfloat16 *sval, const float *u, float *out, SpmvMode mode,
                     const SpmvArgs &a, cudaStream_t s);
@@ -173,7 +173,7 @@ void jacobi_bsr2(const Pattern &P, const double *val, const int *diag, T *dinv, 
 // with x_{k+1} = c0 x_k + c1 x_{k-1} + c2 D^-1 (b - A x_k).
 constexpr int kMaxSmoothDegree = 16;
 // Coarsest multigrid level: a dense FP64 inverse (rebuilt with the level's
-// operator by one thread block) while it has at most kCoarseDenseMax rows or
+// operator) while it has at most kCoarseDenseMax rows or
 // is the singular pressure Laplacian (constant, built once); otherwise
 // kCoarseDegree Chebyshev-Jacobi steps from zero on [hi / kCoarseRatio, hi]
 // (the non-singular blocks are mass-dominated on coarse meshes).

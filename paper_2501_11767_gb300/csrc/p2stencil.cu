@@ -25,7 +25,6 @@ __device__ __forceinline__ typename V2<T>::type mk(T x, T y) {
   return v;
 }
 __device__ __forceinline__ float2 load_pair(const float *p) { return __ldg(reinterpret_cast<const float2 *>(p)); }
-__device__ __forceinline__ double2 load_pair(const double *p) { return __ldg(reinterpret_cast<const double2 *>(p)); }
 __device__ __forceinline__ float2 load_pair(const __nv_bfloat16 *p) {
   return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p));
 }
@@ -283,7 +282,7 @@ __global__ void k_p2_check(int n, int open, const int *__restrict__ rowptr, cons
 
 constexpr int kCount = 2 * (kP2Slots + kP2TopSlots);
 
-bool p2_applies(const Level &L, const P2Table &t, size_t value_size) {
+bool p2_applies(const P2Table &t, size_t value_size) {
   return t.ok && value_size < 8;
 }
 

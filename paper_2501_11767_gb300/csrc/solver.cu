@@ -202,14 +202,7 @@ void MGHier<T>::init(Arena &ar, int kind_, bool singular_, const std::vector<con
     }
     tail_width = wmax <= 8 ? 8 : 16;
     if (tail_l0 > 0 && nl - tail_l0 <= kMaxTailLevels && wmax <= 16) {
-      std::vector<MultiPtr<T>> X(nl), Tt(nl), Rr(nl), B(nl);
-      for (int l = 0; l < nl; ++l) {
-        X[l].p[0] = x[l];
-        Tt[l].p[0] = t[l];
-        Rr[l].p[0] = r[l];
-        B[l].p[0] = b[l];
-      }
-      tail = make_tail(ar, X, Tt, Rr, B);
+      tail = make_tail(ar);
     } else {
       tail_l0 = -1;
     }
@@ -220,8 +213,7 @@ template <typename T>
 static inline const T *transfer_vals(const Transfer &t, bool restrict_);
 
 template <typename T>
-TailDesc<T> *MGHier<T>::make_tail(Arena &ar, const std::vector<MultiPtr<T>> &X, const std::vector<MultiPtr<T>> &Tt,
-                                  const std::vector<MultiPtr<T>> &Rr, const std::vector<MultiPtr<T>> &B) const {
+TailDesc<T> *MGHier<T>::make_tail(Arena &ar) const {
   TailDesc<T> d;
   d.nlev = nl - tail_l0;
   d.degree = degree;
@@ -244,10 +236,10 @@ TailDesc<T> *MGHier<T>::make_tail(Arena &ar, const std::vector<MultiPtr<T>> &X, 
     q.val = val[l];
     q.dinv = dinv[l];
     q.coef = coef[l];
-    q.x = X[l];
-    q.t = Tt[l];
-    q.r = Rr[l];
-    q.b = B[l];
+    q.x = x[l];
+    q.t = t[l];
+    q.r = r[l];
+    q.b = b[l];
     if (l < nl - 1) {
       q.R = view(tr[l]->R);
       q.P = view(tr[l]->P);
@@ -328,14 +320,14 @@ void MGHier<T>::spmv_level(int l, const T *u, T *out, SpmvMode mode, const SpmvA
       return;
     }
     if (bf16) {
-      if (kind == 0) spmv_sell(*pat[l], val16[l], 1, u, out, mode, a, s);
+      if (kind == 0) spmv_sell(*pat[l], val16[l], u, out, mode, a, s);
       else if (kind == 1) spmv_sell_bsr2(*pat[l], val16[l], u, out, mode, a, s);
       else spmv_sell_bsr3(*bpat[l], val16[l], u, out, mode, a, s);
       return;
     }
   }
   if (kind == 0)
-    spmv_sell<T>(*pat[l], val[l], 1, u, out, mode, a, s);
+    spmv_sell<T>(*pat[l], val[l], u, out, mode, a, s);
   else if (kind == 1)
     spmv_sell_bsr2<T>(*pat[l], val[l], u, out, mode, a, s);
   else
@@ -387,10 +379,9 @@ void MGHier<T>::vcycle(int l, cudaStream_t s) {
   const int deg = l == nl - 1 ? kCoarseDegree : degree;
   T *cur = (deg - 1) % 2 == 0 ? x[l] : t[l];
   T *oth = cur == x[l] ? t[l] : x[l];
-  // the P2 stencil forms x_1 on the fly in the two sweeps that read it (in
-  // FP32: one launch and two vector streams less; FP64 sweeps are bound by
-  // their arithmetic, which forming x_1 at every neighbour would double)
-  const bool on_the_fly = stencil(l) && deg > 1 && sizeof(T) == 4;
+  // the P2 stencil forms x_1 on the fly in the two sweeps that read it: one
+  // launch and two vector streams less
+  const bool on_the_fly = stencil(l) && deg > 1;
   if (!on_the_fly) vec_scale_dinv<T>((int)n[l], coef[l], dinv[l], b[l], cur, s);
   for (int k = 1; k < deg; ++k) {
     a.coef = coef[l] + 4 + 3 * (k - 1);
@@ -405,13 +396,13 @@ void MGHier<T>::vcycle(int l, cudaStream_t s) {
   op(l, x[l], r[l], SPMV_RES, ar, s);
   SpmvArgs none;
   if (kind == 1) p2_restrict<T>(p2lev[l + 1]->n, open_top, r[l], b[l + 1], s);
-  else spmv_sell<T>(tr[l]->R, transfer_vals<T>(*tr[l], true), 1, r[l], b[l + 1], SPMV_PLAIN, none, s);
+  else spmv_sell<T>(tr[l]->R, transfer_vals<T>(*tr[l], true), r[l], b[l + 1], SPMV_PLAIN, none, s);
   const int kc = kind == 0 ? Profiler::P1_MG_COARSE : Profiler::VEL_MG_COARSE;
   const int tkc = prof && l == 0 ? prof->start(kc, s) : -1;
   vcycle(l + 1, s);
   if (prof && l == 0) prof->stop(kc, tkc, s, 0.0);   // time only: every level below the finest
   if (kind == 1) p2_prolong_add<T>(p2lev[l + 1]->n, open_top, x[l + 1], x[l], s);
-  else spmv_sell<T>(tr[l]->P, transfer_vals<T>(*tr[l], false), 1, x[l + 1], x[l], SPMV_ADD, none, s);
+  else spmv_sell<T>(tr[l]->P, transfer_vals<T>(*tr[l], false), x[l + 1], x[l], SPMV_ADD, none, s);
   // post-smoothing from x_0 = x[l]
   a.coef = coef[l] + 1;
   a.w = nullptr;
@@ -536,7 +527,7 @@ void MGHier<T>::inner_residual(cudaStream_t s) {
     op(0, acc, b[0], SPMV_RES, a, s);
     dot<double>(n[0], b[0], b[0], ictl + 1, ipartial, s);
   } else {
-    if (kind == 0) spmv_sell<double>(*pat[0], val0_64, 1, acc, r64, SPMV_RES, a, s);
+    if (kind == 0) spmv_sell<double>(*pat[0], val0_64, acc, r64, SPMV_RES, a, s);
     else if (kind == 1) spmv_sell_bsr2<double>(*pat[0], val0_64, acc, r64, SPMV_RES, a, s);
     else spmv_sell_bsr3<double>(*bpat[0], val0_64, acc, r64, SPMV_RES, a, s);
     dot<double>(n[0], r64, r64, ictl + 1, ipartial, s);

@@ -75,14 +75,14 @@ struct MGHier {
   std::vector<const Pattern *> bpat;   // kind 2: node patterns (3x3-block SELL) per level
   std::vector<const int *> bmap;       // kind 2: their map9 (value -> CSR position)
   // kind 1 (set before init): mesh levels (they define the transfers) and
-  // stencil tables; a level that
-  // p2_applies() to is swept as a P2 stencil, any other one as 2x2-block SELL
+  // stencil tables; a level that p2_applies() to is swept as a P2 stencil, any
+  // other one as 2x2-block SELL
   std::vector<const Level *> p2lev;
   std::vector<P2Table> p2tab;
   int open_top = 0;
   VlcPlan vlc;             // coarse end of the FP32 velocity cycle by one cluster
   bool stencil(int l, size_t value_size) const {
-    return kind == 1 && !p2tab.empty() && p2_applies(*p2lev[l], p2tab[l], value_size);
+    return kind == 1 && !p2tab.empty() && p2_applies(p2tab[l], value_size);
   }
   bool stencil(int l) const { return stencil(l, sizeof(T)); }
   std::vector<long> n;
@@ -146,9 +146,8 @@ struct MGHier {
   // inner solves and V-cycles since the last reset, residual ratio of the
   // last solve (stream-ordered read on s, then a synchronisation)
   void inner_stats(bool reset, long long *solves, long long *cycles, double *last_rel, cudaStream_t s);
-  // descriptor of levels tail_l0.. with the given vectors (device copy)
-  TailDesc<T> *make_tail(Arena &ar, const std::vector<MultiPtr<T>> &X, const std::vector<MultiPtr<T>> &Tt,
-                         const std::vector<MultiPtr<T>> &Rr, const std::vector<MultiPtr<T>> &B) const;
+  // descriptor of levels tail_l0.. (device copy)
+  TailDesc<T> *make_tail(Arena &ar) const;
   // out = A_l u with the given epilogue (no profiling)
   void spmv_level(int l, const T *u, T *out, SpmvMode mode, const SpmvArgs &a, cudaStream_t s,
                   P2Start start = P2_PLAIN);

@@ -234,7 +234,7 @@ __global__ void k_sell_gather_t(long nent, int ncomp, const int *__restrict__ ma
   }
 }
 
-template <typename T, typename VT, int NC, bool VEC>
+template <typename T, typename VT>
 __global__ void __launch_bounds__(kSellMaxBlock) k_sell(int nslices, const int *__restrict__ sp, const int *__restrict__ rowid,
                                               const int *__restrict__ col, const VT *__restrict__ val,
                                               const T *__restrict__ u, T *out, int mode, SpmvArgs a) {
@@ -244,29 +244,11 @@ __global__ void __launch_bounds__(kSellMaxBlock) k_sell(int nslices, const int *
   const int b0 = sp[slice], w = (sp[slice + 1] - b0) >> 5;
   const int *cp = col + b0 + lane;
   const VT *vp = val + b0 + lane;
-  T acc0 = 0, acc1 = 0;
+  T acc = 0;
 #pragma unroll 4
-  for (int j = 0; j < w; ++j) {
-    const int c = cp[j * 32];
-    const T v = ldv(vp + j * 32);
-    if (NC == 1) {
-      acc0 += v * u[c];
-    } else if (VEC) {
-      const typename V2t<T>::type x = reinterpret_cast<const typename V2t<T>::type *>(u)[c];
-      acc0 += v * x.x;
-      acc1 += v * x.y;
-    } else {
-      acc0 += v * u[2L * c];
-      acc1 += v * u[2L * c + 1];
-    }
-  }
+  for (int j = 0; j < w; ++j) acc = fma_of((T)ldv(vp + j * 32), u[cp[j * 32]], acc);
   if (row < 0) return;
-  if (NC == 1) {
-    epilogue<T>(mode, row, acc0, u, out, a, a.coef);
-  } else {
-    epilogue<T>(mode, 2L * row, acc0, u, out, a, a.coef);
-    epilogue<T>(mode, 2L * row + 1, acc1, u, out, a, a.coef);
-  }
+  epilogue<T>(mode, row, acc, u, out, a, a.coef);
 }
 
 // Wide rows and few slices (the coarse levels of the 3D velocity hierarchy,
@@ -1523,98 +1505,73 @@ __global__ void __launch_bounds__(kSellMaxBlock) k_sell_w8m(int nslices, const i
 // Every row is computed by the same code as in the per-sweep kernels
 // (sell_w8m_slice, the same scale / copy / dense expressions), so the
 // result is bitwise the multi-launch V-cycle's.
-template <typename T, int NR, int W>
-__device__ void tail_sweep(const TailSell &S, const T *val, const MultiPtr<T> &u, const MultiPtr<T> &out, int mode,
-                           const MultiArgs<T> &a) {
+template <typename T, int W>
+__device__ void tail_sweep(const TailSell &S, const T *val, T *u, T *out, int mode, T *b = nullptr, T *w = nullptr,
+                           const T *dinv = nullptr, const double *coef = nullptr) {
+  MultiPtr<T> um, om;
+  MultiArgs<T> a;
+  um.p[0] = u;
+  om.p[0] = out;
+  a.b.p[0] = b;
+  a.w.p[0] = w;
+  a.dinv = dinv;
+  a.coef = coef;
   const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   for (int slice = threadIdx.x >> 5; slice < S.nslices; slice += nw)
-    sell_w8m_slice<T, NR, W>(slice, lane, S.sp, S.rowid, S.col, val, u, out, mode, a);
+    sell_w8m_slice<T, 1, W>(slice, lane, S.sp, S.rowid, S.col, val, um, om, mode, a);
   __syncthreads();
 }
 
-template <typename T, int NR, int W>
+template <typename T, int W>
 __global__ void __launch_bounds__(512) k_mg_tail(const TailDesc<T> *__restrict__ dp) {
   const TailDesc<T> &d = *dp;
   const int L = d.nlev - 1;
   const int degree = d.degree;
+  // steps of the Chebyshev recurrence from zero, ending in x
+  auto from_zero = [&](const TailLevel<T> &q, int steps) {
+    T *cur = (steps - 1) % 2 == 0 ? q.x : q.t, *oth = cur == q.x ? q.t : q.x;
+    for (int i = threadIdx.x; i < q.n; i += blockDim.x) cur[i] = (T)(*q.coef) * q.dinv[i] * q.b[i];
+    __syncthreads();
+    for (int s = 1; s < steps; ++s) {
+      tail_sweep<T, W>(q.A, q.val, cur, oth, SPMV_CHEB, q.b, s == 1 ? nullptr : oth, q.dinv, q.coef + 4 + 3 * (s - 1));
+      T *const tmp = cur;
+      cur = oth;
+      oth = tmp;
+    }
+  };
   // down: pre-smoothing, residual, restriction
   for (int l = 0; l < L; ++l) {
     const TailLevel<T> &q = d.lv[l];
-    MultiPtr<T> cur = (degree - 1) % 2 == 0 ? q.x : q.t;
-    MultiPtr<T> oth = (degree - 1) % 2 == 0 ? q.t : q.x;
-    for (int i = threadIdx.x; i < q.n; i += blockDim.x)
-      for (int k = 0; k < NR; ++k) cur.p[k][i] = (T)(*q.coef) * q.dinv[i] * q.b.p[k][i];
-    __syncthreads();
-    MultiArgs<T> a;
-    a.b = q.b;
-    a.dinv = q.dinv;
-    for (int s = 1; s < degree; ++s) {
-      a.coef = q.coef + 4 + 3 * (s - 1);
-      a.w = s == 1 ? MultiPtr<T>() : oth;
-      tail_sweep<T, NR, W>(q.A, q.val, cur, oth, SPMV_CHEB, a);
-      const MultiPtr<T> tmp = cur;
-      cur = oth;
-      oth = tmp;
-    }
-    MultiArgs<T> ar;
-    ar.b = q.b;
-    tail_sweep<T, NR, W>(q.A, q.val, q.x, q.r, SPMV_RES, ar);
-    MultiArgs<T> none;
-    tail_sweep<T, NR, W>(q.R, q.Rval, q.r, d.lv[l + 1].b, SPMV_PLAIN, none);
+    from_zero(q, degree);
+    tail_sweep<T, W>(q.A, q.val, q.x, q.r, SPMV_RES, q.b);
+    tail_sweep<T, W>(q.R, q.Rval, q.r, d.lv[l + 1].b, SPMV_PLAIN);
   }
-  // coarsest: dense inverse, or Chebyshev steps from zero (same sweeps as
-  // the pre-smoothing, coarse_degree of them)
+  // coarsest: dense inverse, or Chebyshev steps from zero
   if (d.coarse_degree > 0) {
-    const TailLevel<T> &q = d.lv[L];
-    const int cd = d.coarse_degree;
-    MultiPtr<T> cur = (cd - 1) % 2 == 0 ? q.x : q.t;
-    MultiPtr<T> oth = (cd - 1) % 2 == 0 ? q.t : q.x;
-    for (int i = threadIdx.x; i < q.n; i += blockDim.x)
-      for (int k = 0; k < NR; ++k) cur.p[k][i] = (T)(*q.coef) * q.dinv[i] * q.b.p[k][i];
-    __syncthreads();
-    MultiArgs<T> a;
-    a.b = q.b;
-    a.dinv = q.dinv;
-    for (int st = 1; st < cd; ++st) {
-      a.coef = q.coef + 4 + 3 * (st - 1);
-      a.w = st == 1 ? MultiPtr<T>() : oth;
-      tail_sweep<T, NR, W>(q.A, q.val, cur, oth, SPMV_CHEB, a);
-      const MultiPtr<T> tmp = cur;
-      cur = oth;
-      oth = tmp;
-    }
+    from_zero(d.lv[L], d.coarse_degree);
   } else {
     const TailLevel<T> &q = d.lv[L];
-    for (int r = threadIdx.x; r < d.nc; r += blockDim.x)
-      for (int k = 0; k < NR; ++k) {
-        double s = 0.0;
-        for (int c = 0; c < d.nc; ++c) s = fma(d.cinv[(long)r * d.nc + c], (double)q.b.p[k][c], s);
-        q.x.p[k][r] = (T)s;
-      }
+    for (int r = threadIdx.x; r < d.nc; r += blockDim.x) {
+      double s = 0.0;
+      for (int c = 0; c < d.nc; ++c) s = fma(d.cinv[(long)r * d.nc + c], (double)q.b[c], s);
+      q.x[r] = (T)s;
+    }
     __syncthreads();
   }
   // up: prolongation, post-smoothing
   for (int l = L - 1; l >= 0; --l) {
     const TailLevel<T> &q = d.lv[l];
-    MultiArgs<T> none;
-    tail_sweep<T, NR, W>(q.P, q.Pval, d.lv[l + 1].x, q.x, SPMV_ADD, none);
-    MultiArgs<T> a;
-    a.b = q.b;
-    a.dinv = q.dinv;
-    a.coef = q.coef + 1;
-    tail_sweep<T, NR, W>(q.A, q.val, q.x, q.t, SPMV_CHEB, a);
-    MultiPtr<T> cur = q.t, oth = q.x;
+    tail_sweep<T, W>(q.P, q.Pval, d.lv[l + 1].x, q.x, SPMV_ADD);
+    tail_sweep<T, W>(q.A, q.val, q.x, q.t, SPMV_CHEB, q.b, nullptr, q.dinv, q.coef + 1);
+    T *cur = q.t, *oth = q.x;
     for (int s = 1; s < degree; ++s) {
-      a.coef = q.coef + 4 + 3 * (s - 1);
-      a.w = oth;
-      tail_sweep<T, NR, W>(q.A, q.val, cur, oth, SPMV_CHEB, a);
-      const MultiPtr<T> tmp = cur;
+      tail_sweep<T, W>(q.A, q.val, cur, oth, SPMV_CHEB, q.b, oth, q.dinv, q.coef + 4 + 3 * (s - 1));
+      T *const tmp = cur;
       cur = oth;
       oth = tmp;
     }
-    if (cur.p[0] != q.x.p[0]) {
-      for (int i = threadIdx.x; i < q.n; i += blockDim.x)
-        for (int k = 0; k < NR; ++k) q.x.p[k][i] = cur.p[k][i];
+    if (cur != q.x) {
+      for (int i = threadIdx.x; i < q.n; i += blockDim.x) q.x[i] = cur[i];
       __syncthreads();
     }
   }
@@ -1980,17 +1937,17 @@ void launch_sell_split(const Sell &S, const VT *sval, const T *u, T *out, SpmvMo
 }
 
 template <typename T, typename VT>
-void spmv_sell_impl(const Pattern &P, const VT *sval, int ncomp, const T *u, T *out, SpmvMode mode,
+void spmv_sell_impl(const Pattern &P, const VT *sval, const T *u, T *out, SpmvMode mode,
                     const SpmvArgs &a, cudaStream_t s) {
   const Sell &S = P.sell;
   if (S.nslices == 0) return;
   const int nb = nblocks((long)S.nslices * 32, S.block);
-  const int K = ncomp == 1 && !S.stencil ? sell_split(S) : 1;
-  if (ncomp == 1 && S.stencil) {
+  const int K = S.stencil ? 1 : sell_split(S);
+  if (S.stencil) {
     StencilOff so;
     for (int j = 0; j < 7; ++j) so.o[j] = S.soff[j];
     k_stencil7<T, VT><<<nblocks(P.nrows, S.block), S.block, 0, s>>>(P.nrows, so, sval, u, out, mode, a);
-  } else if (ncomp == 1 && S.wmax <= 8)
+  } else if (S.wmax <= 8)
     k_sell_w8<T, VT><<<nb, S.block, 0, s>>>(S.nslices, S.slice_ptr, S.rowid, S.col, sval, u, out, mode, a);
   else if (K == 2)
     launch_sell_split<T, VT, 2>(S, sval, u, out, mode, a, s);
@@ -2002,12 +1959,8 @@ void spmv_sell_impl(const Pattern &P, const VT *sval, int ncomp, const T *u, T *
     launch_sell_split<T, VT, 16>(S, sval, u, out, mode, a, s);
   else if (K == 32)
     launch_sell_split<T, VT, 32>(S, sval, u, out, mode, a, s);
-  else if (ncomp == 1)
-    k_sell<T, VT, 1, false><<<nb, S.block, 0, s>>>(S.nslices, S.slice_ptr, S.rowid, S.col, sval, u, out, mode, a);
-  else if (aligned(u, 2 * sizeof(T)))
-    k_sell<T, VT, 2, true><<<nb, S.block, 0, s>>>(S.nslices, S.slice_ptr, S.rowid, S.col, sval, u, out, mode, a);
   else
-    k_sell<T, VT, 2, false><<<nb, S.block, 0, s>>>(S.nslices, S.slice_ptr, S.rowid, S.col, sval, u, out, mode, a);
+    k_sell<T, VT><<<nb, S.block, 0, s>>>(S.nslices, S.slice_ptr, S.rowid, S.col, sval, u, out, mode, a);
   CHNSS_LAUNCH_CK();
 }
 
@@ -2128,17 +2081,17 @@ void spmv_sell_bsr2_impl(const Pattern &P, const VT *sval, const T *u, T *out, S
 }
 
 template <typename T>
-void spmv_sell(const Pattern &P, const T *sval, int ncomp, const T *u, T *out, SpmvMode mode, const SpmvArgs &a,
+void spmv_sell(const Pattern &P, const T *sval, const T *u, T *out, SpmvMode mode, const SpmvArgs &a,
                cudaStream_t s) {
-  spmv_sell_impl<T, T>(P, sval, ncomp, u, out, mode, a, s);
+  spmv_sell_impl<T, T>(P, sval, u, out, mode, a, s);
 }
-template void spmv_sell<double>(const Pattern &, const double *, int, const double *, double *, SpmvMode,
+template void spmv_sell<double>(const Pattern &, const double *, const double *, double *, SpmvMode,
                                 const SpmvArgs &, cudaStream_t);
-template void spmv_sell<float>(const Pattern &, const float *, int, const float *, float *, SpmvMode,
+template void spmv_sell<float>(const Pattern &, const float *, const float *, float *, SpmvMode,
                                const SpmvArgs &, cudaStream_t);
-void spmv_sell(const Pattern &P, const __nv_bfloat16 *sval, int ncomp, const float *u, float *out, SpmvMode mode,
+void spmv_sell(const Pattern &P, const __nv_bfloat16 *sval, const float *u, float *out, SpmvMode mode,
                const SpmvArgs &a, cudaStream_t s) {
-  spmv_sell_impl<float, __nv_bfloat16>(P, sval, ncomp, u, out, mode, a, s);
+  spmv_sell_impl<float, __nv_bfloat16>(P, sval, u, out, mode, a, s);
 }
 
 template <typename T>
@@ -2697,8 +2650,8 @@ template void dense_apply_multi<float>(int, int, const double *, const MultiPtr<
 
 template <typename T>
 void mg_tail(const TailDesc<T> *d_desc, int width, cudaStream_t s) {
-  if (width == 8) k_mg_tail<T, 1, 8><<<1, 512, 0, s>>>(d_desc);
-  else if (width == 16) k_mg_tail<T, 1, 16><<<1, 512, 0, s>>>(d_desc);
+  if (width == 8) k_mg_tail<T, 8><<<1, 512, 0, s>>>(d_desc);
+  else if (width == 16) k_mg_tail<T, 16><<<1, 512, 0, s>>>(d_desc);
   else throw Error{CHNSS_ERR_ARG, "coarse-level block: rows of 8 or 16 entries"};
   CHNSS_LAUNCH_CK();
 }

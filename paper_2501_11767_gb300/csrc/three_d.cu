@@ -1512,7 +1512,7 @@ void prec_ch3(chnss3_ctx *c, Prec3<T> &P, int sp, const double *r, double *z, cu
   vec_convert<double, T>(N1, r + N1, X1.input(), s);
   X1.apply(s);
   SpmvArgs none;
-  spmv_sell<T>(c->lv[0].p1, P.Ms, 1, X1.output(), X2.input(), SPMV_PLAIN, none, s);
+  spmv_sell<T>(c->lv[0].p1, P.Ms, X1.output(), X2.input(), SPMV_PLAIN, none, s);
   X2.apply(s);
   mg_output(X2, N1, z + N1, s);
   join3(c, sp, s);
@@ -1527,7 +1527,7 @@ void prec_ns3(chnss3_ctx *c, Prec3<T> &P, const double *r, double *z, cudaStream
   vec_convert<double, T>(N1, r + nv, P.Kp.input(), q);
   P.Kp.apply(q);
   SpmvArgs none;
-  spmv_sell<T>(F.p1, P.Aps, 1, P.Kp.output(), P.mb, SPMV_PLAIN, none, q);
+  spmv_sell<T>(F.p1, P.Aps, P.Kp.output(), P.mb, SPMV_PLAIN, none, q);
   vec_scale_dinv<T>((int)N1, c->massc, P.mdinv, P.mb, P.mx, q);
   SpmvArgs a;
   a.b = P.mb;
@@ -1536,7 +1536,7 @@ void prec_ns3(chnss3_ctx *c, Prec3<T> &P, const double *r, double *z, cudaStream
   for (int k = 1; k <= 4; ++k) {
     a.coef = c->massc + 1 + 3 * (k - 1);
     a.w = k == 1 ? nullptr : other;
-    spmv_sell<T>(F.p1, P.Ms, 1, cur, other, SPMV_CHEB, a, q);
+    spmv_sell<T>(F.p1, P.Ms, cur, other, SPMV_CHEB, a, q);
     std::swap(cur, other);
   }
   vec_convert<T, double>(N1, cur, z + nv, q);
@@ -1620,7 +1620,7 @@ struct AC3Op : LinearOperator {
   long size() const override { return c->lv[0].N1; }
   void apply(const double *x, double *y, cudaStream_t s) override {
     SpmvArgs none;
-    spmv_sell<double>(c->lv[0].p1, c->ACs, 1, x, y, SPMV_PLAIN, none, s);
+    spmv_sell<double>(c->lv[0].p1, c->ACs, x, y, SPMV_PLAIN, none, s);
   }
   void precond(const double *r, double *z, cudaStream_t s) override { run_prec3(c, 3, c->lv[0].N1, r, z, s); }
 };
@@ -1633,8 +1633,8 @@ struct NS3Op : LinearOperator {
     const long nv = 3 * c->lv[0].N2;
     SpmvArgs none;
     spmv_sell_bsr3<double>(c->lv[0].pv3, c->As, x, y, SPMV_PLAIN, none, s);
-    spmv_sell<double>(c->pbt, c->Bts, 1, x + nv, y, SPMV_ADD, none, s);
-    spmv_sell<double>(c->pb, c->Bs, 1, x, y + nv, SPMV_PLAIN, none, s);
+    spmv_sell<double>(c->pbt, c->Bts, x + nv, y, SPMV_ADD, none, s);
+    spmv_sell<double>(c->pb, c->Bs, x, y + nv, SPMV_PLAIN, none, s);
   }
   void precond(const double *r, double *z, cudaStream_t s) override {
     run_prec3(c, 4, 3 * c->lv[0].N2 + c->lv[0].N1, r, z, s);
@@ -1764,7 +1764,7 @@ struct AC3OpT : LinearOperator {
   long size() const override { return c->lv[0].N1; }
   void apply(const double *x, double *y, cudaStream_t s) override {
     SpmvArgs none;
-    spmv_sell<double>(c->lv[0].p1, c->ACsT, 1, x, y, SPMV_PLAIN, none, s);
+    spmv_sell<double>(c->lv[0].p1, c->ACsT, x, y, SPMV_PLAIN, none, s);
   }
   void precond(const double *r, double *z, cudaStream_t s) override { run_prec3(c, 3, c->lv[0].N1, r, z, s); }
 };
@@ -1776,9 +1776,9 @@ struct NS3OpT : LinearOperator {   // [[A^T, B^T], [B, 0]]
   void apply(const double *x, double *y, cudaStream_t s) override {
     const long nv = 3 * c->lv[0].N2;
     SpmvArgs none;
-    spmv_sell<double>(c->lv[0].pv, c->AsT, 1, x, y, SPMV_PLAIN, none, s);
-    spmv_sell<double>(c->pbt, c->Bts, 1, x + nv, y, SPMV_ADD, none, s);
-    spmv_sell<double>(c->pb, c->Bs, 1, x, y + nv, SPMV_PLAIN, none, s);
+    spmv_sell<double>(c->lv[0].pv, c->AsT, x, y, SPMV_PLAIN, none, s);
+    spmv_sell<double>(c->pbt, c->Bts, x + nv, y, SPMV_ADD, none, s);
+    spmv_sell<double>(c->pb, c->Bs, x, y + nv, SPMV_PLAIN, none, s);
   }
   void precond(const double *r, double *z, cudaStream_t s) override {
     run_prec3(c, 4, 3 * c->lv[0].N2 + c->lv[0].N1, r, z, s);

@@ -328,10 +328,7 @@ bool layout(int first, const std::vector<const Level *> &lev, int open, int degr
     q.ld = p2_ld(q.n);
     const bool bare = l == L && !coarse_iter;
     if (q.n > kLargest) return false;
-    if (!bare && q.n > kSerial) {
-      if (q.n < 16) return false;        // fewer than four lines a block
-      d.na = l + 1;
-    }
+    if (!bare && q.n > kSerial) d.na = l + 1;
   }
   ctas = d.na == 0 ? 1 : kVlcCtas;
   if (d.na > 0) {   // even line counts by the coarsest spread level, doubled towards the finer ones
