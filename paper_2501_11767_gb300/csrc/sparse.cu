@@ -434,6 +434,7 @@ __global__ void __launch_bounds__(1024) k_cheb_bsr3_block(int nslices, int K, co
     T acc[3] = {0, 0, 0};
     if (slice < nslices) {
       const int b0 = sp[slice], w = (sp[slice + 1] - b0) >> 5;
+#pragma unroll 2   // two entries' loads at a time: 56 -> 49 us on the 2^3 level
       for (int j = k; j < w; j += K) {
         const int c = col[b0 + j * 32 + lane];
         const VT *vb = val + 9 * (b0 + j * 32) + lane;
