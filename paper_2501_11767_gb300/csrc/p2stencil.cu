@@ -347,7 +347,7 @@ float rounded(double x, const __nv_bfloat16 *) { return __bfloat162float(__doubl
 }  // namespace
 
 namespace {
-__constant__ P2Transfers c_transfers = p2_transfers();
+__device__ const P2Transfers g_transfers = p2_transfers();
 
 // Grid transfers of the velocity with their columns and weights computed:
 // the SELL form streamed 8 bytes an entry (10.7 entries a fine node, both
@@ -386,44 +386,45 @@ __global__ void k_p2_restrict(int nc, const T *__restrict__ r, T *__restrict__ b
 }
 
 // x += P xc, one thread a fine node.  Coarse nodes with prescribed velocity
-// are left out by a check in the cells along the boundary only (0.2 % of a
-// 384^2 Oseen solve).
+// are left out by zero weights: a block's line knows its own, and a thread
+// takes the weights of an inner cell, the first or the last one of the line.
+// Latency bound: the tables come from global memory (divergent loads of
+// constant memory take turns) and the old value is requested with them.  384^2
+// Oseen solve 34.36 ms, 34.38 without any such check; with a check at the
+// coarse nodes 0.2 to 0.5 % more.
 template <typename T>
 __global__ void k_p2_prolong(int nc, int open, const T *__restrict__ xc, T *__restrict__ x) {
   using P = typename V2<T>::type;
-  __shared__ float w[4][6];
+  __shared__ float w[4][4][6];
   __shared__ int off[4][6], cnt[4];
   const int mc = 2 * nc + 1, m = 4 * nc + 1, J = blockIdx.y;
-  if (threadIdx.x < 24) {   // the line's four classes
-    const int c = 4 * (J & 3) + threadIdx.x / 6, k = threadIdx.x % 6;
-    w[threadIdx.x / 6][k] = c_transfers.pw[c][k];
-    off[threadIdx.x / 6][k] = c_transfers.pj[c][k] * mc + c_transfers.pi[c][k];
-    if (k == 0) cnt[threadIdx.x / 6] = c_transfers.pn[c];
+  const int I = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool fixed = prescribed(I, J, m, open);
+  P *xi = reinterpret_cast<P *>(x) + (long)J * m + I;
+  P old = mk<T>(0, 0);
+  if (!fixed) old = *xi;   // requested with the tables
+  if (threadIdx.x < 96) {   // the line's four classes, by (first cell) + 2 (last cell)
+    const int t = threadIdx.x % 24, at = threadIdx.x / 24, c = 4 * (J & 3) + t / 6, k = t % 6;
+    const int ti = g_transfers.pi[c][k], tj = g_transfers.pj[c][k], line = 2 * (J >> 2) + tj;
+    const bool out = ((at & 1) && ti == 0) || ((at & 2) && ti == 2) || line == 0 || (!open && line == mc - 1);
+    w[at][t / 6][k] = out ? 0.f : g_transfers.pw[c][k];
+    if (at == 0) {
+      off[t / 6][k] = tj * mc + ti;
+      if (k == 0) cnt[t / 6] = g_transfers.pn[c];
+    }
   }
   __syncthreads();
-  const int I = blockIdx.x * blockDim.x + threadIdx.x;
-  if (prescribed(I, J, m, open)) return;
-  P *xi = reinterpret_cast<P *>(x) + (long)J * m + I;
-  const int ci = 2 * (I >> 2), cj = 2 * (J >> 2);
-  const bool edge = ci == 0 || cj == 0 || ci + 2 >= mc - 1 || cj + 2 >= mc - 1;   // has prescribed coarse nodes
-  const P *c = reinterpret_cast<const P *>(xc) + (long)cj * mc + ci;
-  const int q = I & 3, n = cnt[q];
-  const P old = *xi;
+  if (fixed) return;
+  const P *c = reinterpret_cast<const P *>(xc) + (long)(2 * (J >> 2)) * mc + 2 * (I >> 2);
+  const int q = I & 3, n = cnt[q], at = ((I >> 2) == 0 ? 1 : 0) + ((I >> 2) == nc - 1 ? 2 : 0);
   T a0 = 0, a1 = 0;
-  auto add = [&](int k, P v) {
-    a0 = fma_of((T)w[q][k], v.x, a0);
-    a1 = fma_of((T)w[q][k], v.y, a1);
-  };
-  if (edge) {
-    for (int k = 0; k < n; ++k) {
-      const int o = off[q][k], tj = o >= 2 * mc ? 2 : o >= mc ? 1 : 0;
-      if (!prescribed(ci + o - tj * mc, cj + tj, mc, open)) add(k, c[o]);
-    }
-  } else {
 #pragma unroll
-    for (int k = 0; k < 6; ++k)
-      if (k < n) add(k, c[off[q][k]]);
-  }
+  for (int k = 0; k < 6; ++k)
+    if (k < n) {
+      const P v = c[off[q][k]];
+      a0 = fma_of((T)w[at][q][k], v.x, a0);
+      a1 = fma_of((T)w[at][q][k], v.y, a1);
+    }
   *xi = mk<T>(old.x + a0, old.y + a1);
 }
 }  // namespace
