@@ -42,10 +42,11 @@ inline long p2_values_count(int n) { return 2 * kP2Slots * p2_ld(n); }   // scal
 // Whether a level of table t takes the stencil for values of value_size
 // bytes: in FP32 and BF16 (384^2: fine level 31.0 -> 18.0 us a sweep, 192^2
 // level 12.1 -> 10.9, coarser ones 6.1 -> 4.4-5.1).  FP64 sweeps stay on the
-// 2x2-block SELL: they are bound by the FP64 pipe, not by the bytes saved, and
-// the stencil's fewer, longer threads keep it less busy (FP64 steps with the
-// stencil from 241^2 on against SELL: 512^2 137 and 131 ms, 768^2 287 and 267,
-// 1024^2 497 and 460; a sweep of 128^2 18.7 and 16.5 us).
+// 2x2-block SELL: they keep the FP64 pipe 73 % (256^2) and 64 % (128^2) busy at
+// 40 and 24 % of HBM, so saved bytes buy little, and the stencil's fewer,
+// longer threads keep it less busy (FP64 steps with the stencil from 241^2 on
+// against SELL: 512^2 137 and 131 ms, 768^2 287 and 267, 1024^2 497 and 460; a
+// sweep of 128^2 18.7 and 16.5 us).
 bool p2_applies(const P2Table &t, size_t value_size);
 // Table of the level's constant blocks A (CSR order, 4 values each) and
 // whether all its rows match it (synchronises s); device copies from keep.
