@@ -390,8 +390,9 @@ __global__ void k_p2_restrict(int nc, const T *__restrict__ r, T *__restrict__ b
 // takes the weights of an inner cell, the first or the last one of the line.
 // Latency bound: the tables come from global memory (divergent loads of
 // constant memory take turns) and the old value is requested with them.  384^2
-// Oseen solve 34.36 ms, 34.38 without any such check; with a check at the
-// coarse nodes 0.2 to 0.5 % more.
+// Oseen solve, against the form that left no node out: 34.36 and 34.38, 34.86
+// and 34.87, 36.35 and 36.18 ms; with a check at the coarse nodes 0.2 to 0.6 %
+// more in every run.
 template <typename T>
 __global__ void k_p2_prolong(int nc, int open, const T *__restrict__ xc, T *__restrict__ x) {
   using P = typename V2<T>::type;
